@@ -883,6 +883,9 @@ def conv_op_bytes(net):
         f, b = algorithmic_bytes(layer.w)
         if net.cols[l] is None:   # direct convolution: reads the input map itself
             out[f"conv_fwd{l}"] = x_bytes + nb(net.W[l]) + nb(net.I[l])
+            if net.direct_scan[l]:   # with its scan and pooling
+                out[f"conv_fwd{l}"] += (nb(layer.spk) + nb(layer.mem) + nb(layer.ckpt)
+                                        + nb(net.pool[l]) + nb(net.idx[l]))
         else:
             out[f"im2col{l}"] = x_bytes + nb(net.cols[l])
             if net.I[l] is None:  # GEMM with the scan in its epilogue
@@ -892,7 +895,8 @@ def conv_op_bytes(net):
                 out[f"conv_fwd{l}"] = nb(net.cols[l]) + nb(net.W[l]) + nb(net.I[l])
         if net.I[l] is not None:
             out[f"scan_fwd{l}"] = f * ns
-        out[f"pool_fwd{l}"] = nb(layer.spk) + nb(net.pool[l]) + nb(net.idx[l])
+        if not net.direct_scan[l]:
+            out[f"pool_fwd{l}"] = nb(layer.spk) + nb(net.pool[l]) + nb(net.idx[l])
         out[f"pool_bwd{l}"] = nb(net.grad_pool[l]) + nb(net.idx[l]) + nb(net.grad_spk[l])
         out[f"scan_bwd{l}"] = b * ns
         src = x_bytes if net.cols[l] is None else nb(net.cols[l])

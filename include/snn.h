@@ -483,6 +483,30 @@ snn_status_t snn_conv2d_small_dw_nhwc(int64_t M, int64_t H, int64_t W, int64_t C
                                       snn_stream_t stream);
 
 /*
+ * First-layer convolution with its Leaky scan and 2x2 max pooling in one
+ * kernel (the CSNN's 5x5 filters over the 1-channel input map; Eqs. 3-4):
+ * the same results as snn_conv2d_small_fwd_nhwc, snn_leaky_fwd and
+ * snn_maxpool2_fwd_nhwc in turn wherever the currents' sums are exact in
+ * fp32 (spikes times bf16 filters), else within fp32 rounding of the
+ * currents; the currents are never written.
+ *   desc     the Leaky layer: B, N = Ho*Wo*Cout (channel-last), io_dtype
+ *            SNN_BF16, save SNN_SAVE_MEM, any reset; beta_mode and thr_mode
+ *            scalar or per channel with C = Cout, HW = 1
+ *   X        bf16 [T*B, H, W, 1];  Wt bf16 [Cout, ldw] as above
+ *   spk, mem bf16 [T, B, N] (out);  ckpt the spike bits, or NULL
+ *   pool     bf16 [T*B, Ho/2, Wo/2, Cout] (out) and idx uint8 (out): the
+ *            pooled spikes and positions, or both NULL
+ * Cin = 1, KH = KW of 3 or 5, Cout = 16, Ho and Wo even, H*W a multiple
+ * of 8 and at most 8192; SNN_ERR_UNSUPPORTED otherwise.  Initial state zero.
+ */
+snn_status_t snn_conv2d_small_leaky_fwd_nhwc(const snn_scan_desc* desc, int64_t H, int64_t W,
+                                             int64_t Cin, int64_t Cout, int64_t KH, int64_t KW,
+                                             int64_t ldw, const void* X, const void* Wt,
+                                             const float* beta, const float* thr, void* spk,
+                                             void* mem, float* ckpt, void* pool, uint8_t* idx,
+                                             snn_stream_t stream);
+
+/*
  * AdamW update of n fp32 master weights (the optimiser of the paper's
  * training runs, Sec. V; decoupled weight decay):
  *   m <- beta1 m + (1 - beta1) g ;  v <- beta2 v + (1 - beta2) g^2

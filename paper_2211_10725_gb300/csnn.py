@@ -31,7 +31,8 @@ padded to 32).
 it instead of recomputing from the currents) and runs the GEMM layers (the
 second convolution over its patch rows, the readout) as one kernel each:
 the GEMM with the Leaky scan in its epilogue, so their currents never
-reach HBM.
+reach HBM; the first layer's direct convolution likewise carries its scan and
+its pooling.
 """
 from __future__ import annotations
 
@@ -79,6 +80,11 @@ class ConvSNN:
         g0 = self.geo[0]
         self.direct = [direct_first and g0[4] * g0[4] * g0[2] <= 32 and g0[3] <= 16
                        and g0[0] * g0[1] * g0[2] <= 8192] + [False] * (len(self.geo) - 1)
+        # ... and, with the traces stored, in one kernel with its scan and pooling
+        # (the shapes snn_conv2d_small_leaky_fwd_nhwc takes)
+        self.direct_scan = [self.fused and d and g[2] == 1 and g[4] in (3, 5) and g[3] == 16
+                            and g[5] % 2 == 0 and g[6] % 2 == 0 and g[0] * g[1] % 8 == 0
+                            for d, g in zip(self.direct, self.geo)]
         self.n_out = _pad8(w.n_classes)
 
         # weights: one flat buffer per quantity, each block on a 64-element
@@ -135,7 +141,8 @@ class ConvSNN:
         for l, (h, wd, cin, cout, k, ho, wo, hp, wp, kpad) in enumerate(self.geo):
             rows = M * ho * wo
             self.cols.append(None if self.direct[l] else torch.empty((rows, kpad), **bf))
-            fuse = self.fused and not self.direct[l]  # GEMM and scan in one kernel
+            # convolution (or GEMM) and scan in one kernel: no currents
+            fuse = self.fused and (not self.direct[l] or self.direct_scan[l])
             self.I.append(None if fuse else
                           torch.empty((rows, cout), dtype=torch.float32, device=dev))
             lw = W.ScanWorkload(name=f"csnn_conv{l}", neuron="leaky", T=T, B=B,
@@ -190,6 +197,13 @@ class ConvSNN:
         out = []
         for l, (h, wd, cin, cout, k, ho, wo, hp, wp, kpad) in enumerate(self.geo):
             layer = self.layers[l]
+            if self.direct_scan[l]:  # convolution, scan and pooling in one kernel
+                out.append((f"conv_fwd{l}", lambda l=l, layer=layer, k=k:
+                            snn.snn_conv2d_small_leaky_fwd_nhwc(
+                                layer.desc, self.layer_input(l, X), self.W[l], self.beta[l],
+                                self.thr, layer.spk, layer.mem, layer.ckpt, self.pool[l],
+                                self.idx[l], k, k, stream)))
+                continue
             if self.direct[l]:
                 out.append((f"conv_fwd{l}", lambda l=l, k=k, s=(M, ho, wo, cout):
                             snn.snn_conv2d_small_fwd_nhwc(self.layer_input(l, X), self.W[l],

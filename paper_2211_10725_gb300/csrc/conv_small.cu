@@ -18,7 +18,7 @@
 #include <climits>
 #include <cstdint>
 
-#include "launch.cuh"
+#include "scan_host.cuh"
 #include "snn.h"
 
 namespace snn {
@@ -515,22 +515,220 @@ __global__ void __maxnreg__(96) conv_slide_dw_kernel(
   }
 }
 
-// dW[o, k] = sum of the G block partials, 0 for k >= K: one warp per
-// output, lane l adding partials l, l + 32, ... in order, then a fixed
-// shuffle tree over the lanes.
-__global__ void conv_small_dw_sum(const float* __restrict__ part, float* __restrict__ dW, int G,
-                                  int Cout, int K, int ldw) {
+// ---- Weight gradient on the tensor cores: one input channel, 5x5 or 3x3 --
+//
+// dW[o, k] = sum over pixels p of dI[p, o] * X[p + tap k] is a product with
+// M = Cout, N = KH*KW and the pixels of every image as its reduction: 16
+// pixels per mma (m16n8k16), four column blocks for 25 taps.  Both operands
+// come straight from the raw bf16 images in shared memory: A = dI^T through
+// ldmatrix.trans (dI is [pixel][channel]), and a B register is two
+// neighbouring pixels' values of one tap, i.e. two neighbouring elements of
+// an image row (one or two words and a byte permute, by the tap's parity;
+// the output width is even, so a pixel pair never straddles two rows).
+// M = 16 is an eighth of the smallest tcgen05 tile, so mma.sync it is; the
+// kernel is bound by reading dI (2*Cout bytes a pixel) and by the latency of
+// a block's few images.  The sliding-window FMA kernel above issued 3.7
+// instructions per paired FMA and took 52 us serialised at T = 25, B = 128,
+// [24, 24, 16] (64 MB: 9.4 us at 6.8 TB/s); this kernel takes 25 us there
+// (63% of issue slots), and its error against a float64 sum is the FMA
+// kernel's (8.2e-8 against 8.1e-8 of the result's norm).
+//
+// A block sums images b, b + G, ...; warp w takes pixel groups w, w + 9,
+// ... of each; the warps are added in order into the block partial, so the
+// result is the same on every call.  Images arrive by cp.async, kMmaDwStages
+// - 1 of them in flight ahead of the one being summed.
+constexpr int kMmaDwWarps = 9;  // 36 groups of the CSNN's map: 4 each
+constexpr int kMmaDwThreads = 32 * kMmaDwWarps;
+constexpr int kMmaDwStages = 3;
+static_assert(kMmaDwWarps == 9, "the warps are added three by three");
+
+__device__ __forceinline__ void mma_bf16_zero(float (&d)[4], const uint32_t (&a)[4], uint32_t b0,
+                                              uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
+      "{%8, %9}, {%10, %10, %10, %10};"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.0f));
+}
+
+// Bytes of one staged image: dI, then X and a word past its end, then (once
+// per block, after the stages) a 16-byte row of zeros.
+__host__ __device__ inline int mma_dw_stage_bytes(int pix, int img) {
+  return pix * 2 + (img * 2 + 16);
+}
+
+template <int KS, int COUT>
+__global__ void __launch_bounds__(kMmaDwThreads, 3) conv_mma_dw_kernel(
+    const __nv_bfloat16* __restrict__ X, const __nv_bfloat16* __restrict__ dI,
+    float* __restrict__ part, int64_t M, int H, int W) {
+  constexpr int KK = KS * KS, NBL = (KK + 7) / 8;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  const int Ho = H - KS + 1, Wo = W - KS + 1, P = Ho * Wo;
+  const int img = H * W, pix = P * COUT;
+  const int sbytes = mma_dw_stage_bytes(pix, img);
+  const int t = threadIdx.x, warp = t >> 5, lid = t & 31, g = lid >> 2, q = lid & 3;
+  const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(dsm));
+  const uint32_t zrow = base + kMmaDwStages * sbytes;
+  if (t < 4) reinterpret_cast<uint32_t*>(dsm + kMmaDwStages * sbytes)[t] = 0;
+  const int64_t G = gridDim.x;
   grid_dep_wait();
-  const int e = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (e >= Cout * ldw) return;  // warp-uniform
+  auto stage = [&](int64_t m, int b) {
+    if (m < M) {
+      const unsigned char* gd = reinterpret_cast<const unsigned char*>(dI + m * pix);
+      const unsigned char* gx = reinterpret_cast<const unsigned char*>(X + m * img);
+      unsigned char* s = dsm + b * sbytes;
+      for (int c = t; c < pix / 8; c += kMmaDwThreads) cp_async16(s + 16 * c, gd + 16 * c);
+      for (int c = t; c < img / 8; c += kMmaDwThreads) cp_async16(s + pix * 2 + 16 * c, gx + 16 * c);
+    }
+    cp_async_commit();  // an empty group keeps the wait count uniform
+  };
+  // the tap of B column n = 8*nb + g: byte offset of its word from the pixel
+  // pair's, and the permute that takes its two elements (odd taps straddle)
+  uint32_t toff[NBL], tsel[NBL];
+#pragma unroll
+  for (int nb = 0; nb < NBL; ++nb) {
+    const int k = 8 * nb + g, ky = k / KS, kx = k - ky * KS;
+    const int off = k < KK ? ky * W + kx : 0;  // padding columns repeat tap 0
+    toff[nb] = 4u * (uint32_t)(off >> 1);
+    tsel[nb] = (off & 1) ? 0x5432u : 0x3210u;
+  }
+  float acc[NBL][4];
+#pragma unroll
+  for (int nb = 0; nb < NBL; ++nb) acc[nb][0] = acc[nb][1] = acc[nb][2] = acc[nb][3] = 0.0f;
+  // this lane's A row within a group (ldmatrix address) and its B pixels
+  const int arow = (lid & 7) + (COUT == 16 ? (lid >> 4) * 8 : ((lid >> 3) & 1) * 8);
+  const int acol = COUT == 16 ? ((lid >> 3) & 1) * 8 : 0;
+  const int step_y = 16 * kMmaDwWarps / Wo, step_x = 16 * kMmaDwWarps - step_y * Wo;
+  const int p_first = 16 * warp + 2 * q;
+  const int y_first = p_first / Wo, x_first = p_first - y_first * Wo;
+  const int p8 = p_first + 8;
+  const int y8_first = p8 / Wo, x8_first = p8 - y8_first * Wo;
+  for (int i = 0; i < kMmaDwStages - 1; ++i) stage(blockIdx.x + i * G, i);
+  int i = 0;
+  for (int64_t m = blockIdx.x; m < M; m += G, ++i) {
+    const int b = i % kMmaDwStages;
+    asm volatile("cp.async.wait_group %0;" ::"n"(kMmaDwStages - 2) : "memory");
+    __syncthreads();  // image m has landed for every thread; image i - 1 is no longer read
+    stage(m + (kMmaDwStages - 1) * G, (i + kMmaDwStages - 1) % kMmaDwStages);
+    const uint32_t sd = base + b * sbytes, sx = sd + pix * 2;
+    int y0 = y_first, x0 = x_first, y1 = y8_first, x1 = x8_first;
+    for (int p0 = 16 * warp; p0 < P; p0 += 16 * kMmaDwWarps) {
+      uint32_t a[4] = {0u, 0u, 0u, 0u};
+      const uint32_t ad = p0 + arow < P ? sd + (uint32_t)((p0 + arow) * COUT + acol) * 2 : zrow;
+      if constexpr (COUT == 16) {
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]) : "r"(ad));
+      } else {
+        asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];"
+                     : "=r"(a[0]), "=r"(a[2]) : "r"(ad));
+      }
+      const bool in0 = p0 + 2 * q < P, in1 = p0 + 2 * q + 8 < P;  // P is even
+      const uint32_t w0 = sx + (in0 ? 2u * (uint32_t)(y0 * W + x0) : 0u);
+      const uint32_t w1 = sx + (in1 ? 2u * (uint32_t)(y1 * W + x1) : 0u);
+#pragma unroll
+      for (int nb = 0; nb < NBL; ++nb) {
+        uint32_t l0, h0, l1, h1;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(l0) : "r"(w0 + toff[nb]));
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(h0) : "r"(w0 + toff[nb] + 4));
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(l1) : "r"(w1 + toff[nb]));
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(h1) : "r"(w1 + toff[nb] + 4));
+        uint32_t b0 = __byte_perm(l0, h0, tsel[nb]), b1 = __byte_perm(l1, h1, tsel[nb]);
+        if (!in0) b0 = 0;  // pixels past the map add 0 * 0
+        if (!in1) b1 = 0;
+        // from zero, then a rounded fp32 addition: the tensor core truncates
+        // its sums, and a chain of them over the images showed it (1.4e-7 of
+        // the result's norm at 3200 images, against 8e-8 for fp32 FMAs)
+        float d[4];
+        mma_bf16_zero(d, a, b0, b1);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) acc[nb][r] += d[r];
+      }
+      y0 += step_y;
+      x0 += step_x;
+      if (x0 >= Wo) { x0 -= Wo; ++y0; }
+      y1 += step_y;
+      x1 += step_x;
+      if (x1 >= Wo) { x1 -= Wo; ++y1; }
+    }
+  }
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();  // the stages are free: warp sums, then the block's in warp order
+  float* red = reinterpret_cast<float*>(dsm);  // [warp][COUT][8*NBL]
+#pragma unroll
+  for (int nb = 0; nb < NBL; ++nb)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int o = g + 8 * (r >> 1), n = 8 * nb + 2 * q + (r & 1);
+      if (o < COUT) red[(warp * COUT + o) * (8 * NBL) + n] = acc[nb][r];
+    }
+  __syncthreads();
+  for (int e = t; e < COUT * KK; e += kMmaDwThreads) {
+    const int o = e / KK, k = e - o * KK;
+    float s[3];  // three runs of three warps, then their sum
+#pragma unroll
+    for (int w = 0; w < 3; ++w) {
+      const float* r = red + ((3 * w) * COUT + o) * (8 * NBL) + k;
+      s[w] = (r[0] + r[COUT * 8 * NBL]) + r[2 * COUT * 8 * NBL];
+    }
+    part[(int64_t)blockIdx.x * COUT * KK + e] = (s[0] + s[1]) + s[2];
+  }
+}
+
+// Shapes of the tensor-core weight gradient: an even output width (a pixel
+// pair within one row), whole 16-byte pieces per image, and room for the
+// stages (or, later, the warp sums) in shared memory; one block per SM must
+// fit, three is what the CSNN's [24, 24, 16] takes (60 KB each).
+bool mma_dw_ok(int64_t H, int64_t W, int64_t Cin, int64_t Cout, int64_t KH, int64_t KW, const void* X,
+               const void* dI, size_t* smem) {
+  if (Cin != 1 || KH != KW || (KH != 3 && KH != 5) || (Cout != 8 && Cout != 16)) return false;
+  const int64_t Ho = H - KH + 1, Wo = W - KW + 1;
+  if (Wo % 2 != 0 || (H * W) % 8 != 0 || (Ho * Wo * Cout) % 8 != 0) return false;
+  if ((reinterpret_cast<uintptr_t>(X) | reinterpret_cast<uintptr_t>(dI)) & 15u) return false;
+  const size_t ring = (size_t)kMmaDwStages * mma_dw_stage_bytes((int)(Ho * Wo * Cout), (int)(H * W)) + 16;
+  const size_t sums = (size_t)kMmaDwWarps * Cout * 32 * sizeof(float);
+  *smem = ring > sums ? ring : sums;
+  return *smem <= 220 * 1024;
+}
+
+template <int KS, int COUT>
+cudaError_t launch_mma_dw(const __nv_bfloat16* X, const __nv_bfloat16* dI, float* part, int64_t M,
+                          int H, int W, int64_t G, size_t smem, cudaStream_t st) {
+  const cudaError_t e = ensure_smem((const void*)conv_mma_dw_kernel<KS, COUT>, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(conv_mma_dw_kernel<KS, COUT>, dim3((unsigned)G), dim3(kMmaDwThreads), smem, st, X, dI,
+                    part, M, H, W);
+}
+
+// dW[o, k] = sum of the G block partials, 0 for k >= K: a block takes 32
+// consecutive outputs (coalesced rows of the partials), warp w adds partials
+// w, w + 32, ... in order, then the warps are added in a fixed tree.
+constexpr int kDwSumWarps = 32;
+__global__ void __launch_bounds__(32 * kDwSumWarps) conv_small_dw_sum(
+    const float* __restrict__ part, float* __restrict__ dW, int G, int Cout, int K, int ldw) {
+  __shared__ float sh[kDwSumWarps][32];
+  grid_dep_wait();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int e = blockIdx.x * 32 + lane;
   const int o = e / ldw, k = e - o * ldw;
   float s = 0.0f;
-  if (k < K)
-    for (int b = lane; b < G; b += 32) s += part[((int64_t)b * Cout + o) * K + k];
+  if (o < Cout && k < K) {
+    const float* p = part + o * K + k;
+    const int64_t stride = (int64_t)Cout * K;
+#pragma unroll 8
+    for (int b = warp; b < G; b += kDwSumWarps) s += p[b * stride];
+  }
+  sh[warp][lane] = s;
+  __syncthreads();
+  if (warp == 0 && o < Cout) {
+    float r[kDwSumWarps];
 #pragma unroll
-  for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-  if (lane == 0) dW[e] = s;
+    for (int w = 0; w < kDwSumWarps; ++w) r[w] = sh[w][lane];
+#pragma unroll
+    for (int d = kDwSumWarps / 2; d > 0; d >>= 1)
+#pragma unroll
+      for (int w = 0; w < d; ++w) r[w] += r[w + d];
+    dW[e] = r[0];
+  }
 }
 
 snn_status_t check_small(int64_t M, int64_t H, int64_t W, int64_t Cin, int64_t Cout, int64_t KH,
@@ -664,7 +862,20 @@ extern "C" snn_status_t snn_conv2d_small_dw_nhwc(int64_t M, int64_t H, int64_t W
   const int64_t G = dw_blocks(M, H, W, Cin, Cout, KH, KW);
   float* part = static_cast<float*>(ws);
   cudaError_t e = cudaSuccess;
-  size_t slide_smem = 0;
+  size_t slide_smem = 0, mma_smem = 0;
+  if (mma_dw_ok(H, W, Cin, Cout, KH, KW, X, dI, &mma_smem)) {
+    const __nv_bfloat16* x2 = static_cast<const __nv_bfloat16*>(X);
+    const __nv_bfloat16* d2 = static_cast<const __nv_bfloat16*>(dI);
+    const int h = (int)H, w = (int)W;
+    if (KH == 5) e = Cout == 16 ? launch_mma_dw<5, 16>(x2, d2, part, M, h, w, G, mma_smem, st)
+                                : launch_mma_dw<5, 8>(x2, d2, part, M, h, w, G, mma_smem, st);
+    else e = Cout == 16 ? launch_mma_dw<3, 16>(x2, d2, part, M, h, w, G, mma_smem, st)
+                        : launch_mma_dw<3, 8>(x2, d2, part, M, h, w, G, mma_smem, st);
+    if (e != cudaSuccess) return SNN_ERR_CUDA;
+    e = launch_pdl(conv_small_dw_sum, dim3((unsigned)((Cout * ldw + 31) / 32)), dim3(32 * kDwSumWarps),
+                   0, st, static_cast<const float*>(part), dW, (int)G, (int)Cout, K, (int)ldw);
+    return e == cudaSuccess ? SNN_OK : SNN_ERR_CUDA;
+  }
   if (slide_dw_ok(H, W, Cin, Cout, KH, KW, &slide_smem)) {
     const int thr = ((int)((H - KH + 1) * (Cout / 2)) + 31) / 32 * 32;
     // raw 16-byte copies of whole images: both image sizes a multiple of 8
@@ -683,9 +894,8 @@ extern "C" snn_status_t snn_conv2d_small_dw_nhwc(int64_t M, int64_t H, int64_t W
                 : launch_pdl(conv_slide_dw_kernel<3, 3>, dim3((unsigned)G), dim3(thr), slide_smem, st, x1,
                              d1, part, M, (int)H, (int)W, (int)Cout, vec1);
     if (e != cudaSuccess) return SNN_ERR_CUDA;
-    const int n = (int)(Cout * ldw);  // one warp each
-    e = launch_pdl(conv_small_dw_sum, dim3((unsigned)((n + 7) / 8)), dim3(256), 0, st,
-                   static_cast<const float*>(part), dW, (int)G, (int)Cout, K, (int)ldw);
+    e = launch_pdl(conv_small_dw_sum, dim3((unsigned)((Cout * ldw + 31) / 32)), dim3(32 * kDwSumWarps),
+                   0, st, static_cast<const float*>(part), dW, (int)G, (int)Cout, K, (int)ldw);
     return e == cudaSuccess ? SNN_OK : SNN_ERR_CUDA;
   }
   const int P = (int)((H - KH + 1) * (W - KW + 1));
@@ -715,8 +925,7 @@ extern "C" snn_status_t snn_conv2d_small_dw_nhwc(int64_t M, int64_t H, int64_t W
     e = launch_pdl(conv_small_dw_kernel<0, 0, 0, 32>, dim3((unsigned)G), dim3(kDwThreads), smem, st,
                    x, d, part, M, (int)H, (int)W, (int)Cin, (int)Cout, (int)KH, (int)KW, vec);
   if (e != cudaSuccess) return SNN_ERR_CUDA;
-  const int n = (int)(Cout * ldw);  // one warp each
-  e = launch_pdl(conv_small_dw_sum, dim3((unsigned)((n + 7) / 8)), dim3(256), 0, st,
-                 static_cast<const float*>(part), dW, (int)G, (int)Cout, K, (int)ldw);
+  e = launch_pdl(conv_small_dw_sum, dim3((unsigned)((Cout * ldw + 31) / 32)), dim3(32 * kDwSumWarps), 0,
+                 st, static_cast<const float*>(part), dW, (int)G, (int)Cout, K, (int)ldw);
   return e == cudaSuccess ? SNN_OK : SNN_ERR_CUDA;
 }

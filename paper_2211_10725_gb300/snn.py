@@ -86,6 +86,8 @@ _SIGS = {
     "snn_conv2d_small_dw_workspace_bytes": ([ctypes.c_int64] * 7, ctypes.c_size_t),
     "snn_conv2d_small_dw_nhwc": ([ctypes.c_int64] * 8 + [_P] * 4 + [ctypes.c_size_t, _P],
                                  ctypes.c_int),
+    "snn_conv2d_small_leaky_fwd_nhwc": ([ctypes.POINTER(ScanDesc)] + [ctypes.c_int64] * 7 + [_P] * 10,
+                                        ctypes.c_int),
     "snn_im2col_nhwc": ([ctypes.c_int64] * 7 + [_P] * 3, ctypes.c_int),
     "snn_col2im_nhwc": ([ctypes.c_int64] * 7 + [_P] * 3, ctypes.c_int),
     "snn_maxpool2_fwd_nhwc": ([ctypes.c_int64] * 4 + [_P] * 4, ctypes.c_int),
@@ -413,6 +415,19 @@ def snn_conv2d_small_dw_nhwc(X, dI, dW, KH, KW, ws, stream=None):
                                                    _ptr(dI), _ptr(dW), _ptr(ws),
                                                    ws.numel() * ws.element_size(),
                                                    _stream(stream)), "snn_conv2d_small_dw_nhwc")
+
+
+def snn_conv2d_small_leaky_fwd_nhwc(desc, X, Wt, beta, thr, spk, mem, ckpt, pool, idx, KH, KW,
+                                    stream=None):
+    """Convolution of X [T*B, H, W, 1] with filters Wt [Cout, ldw], the Leaky
+    scan of its currents and the 2x2 max pooling of its spikes (unless pool
+    and idx are None) in one kernel; writes spk, mem (and the spike bits)."""
+    _, H, W_, Cin = X.shape
+    Cout, ldw = Wt.shape
+    _check(load_library().snn_conv2d_small_leaky_fwd_nhwc(
+        ctypes.byref(desc), H, W_, Cin, Cout, KH, KW, ldw, _ptr(X), _ptr(Wt), _ptr(beta),
+        _ptr(thr), _ptr(spk), _ptr(mem), _ptr(ckpt), _ptr(pool), _ptr(idx), _stream(stream)),
+        "snn_conv2d_small_leaky_fwd_nhwc")
 
 
 def snn_im2col_nhwc(X, cols, KH, KW, stream=None):
