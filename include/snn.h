@@ -281,7 +281,7 @@ snn_status_t snn_dense_layer_fwd(int64_t M, int64_t K, int64_t N, const void* X,
  * when dW's few output tiles would each sum a long M (a convolution's
  * weight gradient sums over every patch row), S fp32 partial copies of dW
  * [N, K]: the rows are split S ways, S a function of (M, K, N) alone, and
- * the partials are added in split order (the same bits on every call). */
+ * the partials are added in a fixed order (the same bits on every call). */
 size_t snn_dense_workspace_bytes(int64_t M, int64_t K, int64_t N);
 
 /*

@@ -19,7 +19,7 @@
 #include <climits>
 #include <cstdint>
 
-#include "launch.cuh"
+#include "scan_host.cuh"
 #include "snn.h"
 
 namespace snn {
@@ -177,24 +177,33 @@ __global__ void __launch_bounds__(kThreads) im2col_vec8_kernel(const uint4* __re
   cols[i] = v;
 }
 
-// As im2col_vec8_kernel, kIm2colPer vectors per thread (a block's threads
-// stride over consecutive vectors, so stores stay coalesced and each thread
-// has several loads in flight), the tap of each column group read from a
-// shared-memory table instead of being divided out per element.
-constexpr int kIm2colPer = 4;
+// As im2col_vec8_kernel for any number of patch rows whose column groups fit
+// a table: a block writes a run of consecutive patch rows (about
+// kIm2colBlockVecs vectors), and both halves of a vector's source address,
+// the patch row's first pixel and the column group's tap, come from
+// shared-memory tables that the block fills once.  The row and group of a
+// thread's next vector follow from the last one's by an addition, so a
+// vector costs no division: with three per vector the kernel was bound by
+// issue slots (42 us for the 164 MB of the CSNN's second layer at M = 3200,
+// 64 rows of 400 columns; 24 us at 6.8 TB/s), now 31 us.
 constexpr int kIm2colMaxGroups = 4096;  // column groups (Kpad / 8) the table holds
+constexpr int kIm2colBlockVecs = 4096;
+constexpr int kIm2colMaxRows = 1024;
+constexpr int kIm2colPer = 4;  // vectors a thread loads before it stores them
 
 template <typename Ix>
-__global__ void __launch_bounds__(kThreads) im2col_vec8_multi_kernel(const uint4* __restrict__ X,
-                                                                     uint4* __restrict__ cols,
-                                                                     Ix rows, int H, int W,
-                                                                     int Cin, int KH, int KW,
-                                                                     int Kpad) {
-  __shared__ int toff[kIm2colMaxGroups];  // input offset (16-byte units) of group j's tap, or -1
+__global__ void __launch_bounds__(kThreads) im2col_rows_kernel(const uint4* __restrict__ X,
+                                                               uint4* __restrict__ cols, Ix rows,
+                                                               int H, int W, int Cin, int KH, int KW,
+                                                               int Kpad, int block_rows) {
+  extern __shared__ __align__(16) unsigned char sm[];
   const int Ho = H - KH + 1, Wo = W - KW + 1;
-  const int G = Cin / 8;
-  const int vpr = Kpad / 8;
-  for (int j = threadIdx.x; j < vpr; j += blockDim.x) {
+  const int G = Cin / 8, vpr = Kpad / 8;
+  Ix* row0 = reinterpret_cast<Ix*>(sm);                   // first pixel of row r (16-byte units)
+  int* toff = reinterpret_cast<int*>(row0 + block_rows);  // offset of group j's tap, or -1
+  const Ix r_lo = (Ix)blockIdx.x * block_rows;
+  const int nr = (int)min((Ix)block_rows, rows - r_lo);
+  for (int j = threadIdx.x; j < vpr; j += kThreads) {
     int t = -1;
     if (j < KH * KW * G) {
       const int tap = j / G, g = j - tap * G;
@@ -203,30 +212,37 @@ __global__ void __launch_bounds__(kThreads) im2col_vec8_multi_kernel(const uint4
     }
     toff[j] = t;
   }
+  for (int r = threadIdx.x; r < nr; r += kThreads) {
+    const Ix m = (r_lo + r) / (Ho * Wo);
+    const int p = (int)(r_lo + r - m * (Ho * Wo));
+    const int oy = p / Wo, ox = p - oy * Wo;
+    row0[r] = ((m * H + oy) * W + ox) * G;
+  }
   __syncthreads();
   grid_dep_wait();
-  const Ix total = rows * vpr;
-  const Ix base = (Ix)blockIdx.x * blockDim.x * kIm2colPer + threadIdx.x;
-  uint4 v[kIm2colPer];
+  const int dr = kThreads / vpr, dj = kThreads - dr * vpr;
+  int r = threadIdx.x / vpr, j = threadIdx.x - r * vpr;
+  uint4* out = cols + r_lo * vpr;
+  const int n = nr * vpr;
+  for (int i = threadIdx.x; i < n; i += kIm2colPer * kThreads) {
+    uint4 v[kIm2colPer];
 #pragma unroll
-  for (int u = 0; u < kIm2colPer; ++u) {
-    const Ix i = base + (Ix)u * blockDim.x;
-    v[u] = make_uint4(0u, 0u, 0u, 0u);
-    if (i < total) {
-      const Ix r = i / vpr;
-      const int t = toff[(int)(i - r * vpr)];
-      if (t >= 0) {
-        const Ix m = r / (Ho * Wo);
-        const int p = (int)(r - m * (Ho * Wo));
-        const int oy = p / Wo, ox = p - oy * Wo;
-        v[u] = X[((m * H + oy) * W + ox) * G + t];
+    for (int u = 0; u < kIm2colPer; ++u) {
+      v[u] = make_uint4(0u, 0u, 0u, 0u);
+      if (r < nr) {
+        const int t = toff[j];
+        if (t >= 0) v[u] = __ldg(X + row0[r] + t);
+      }
+      r += dr;
+      j += dj;
+      if (j >= vpr) {
+        j -= vpr;
+        ++r;
       }
     }
-  }
 #pragma unroll
-  for (int u = 0; u < kIm2colPer; ++u) {
-    const Ix i = base + (Ix)u * blockDim.x;
-    if (i < total) cols[i] = v[u];
+    for (int u = 0; u < kIm2colPer; ++u)
+      if (i + u * kThreads < n) out[i + u * kThreads] = v[u];
   }
 }
 
@@ -293,6 +309,94 @@ __global__ void __launch_bounds__(kThreads) col2im_vec8_kernel(const uint4* __re
 #pragma unroll
   for (int e = 0; e < 8; ++e) o.h[e] = __float2bfloat16_rn(s[e]);
   dX[i] = o.u;
+}
+
+// As col2im_vec8_kernel with an image's patch rows staged whole in shared
+// memory: its 25 (or 9) taps of 32 bytes per pixel are scattered over rows
+// 2*Kpad bytes apart, which as direct loads kept 16 sectors per request in
+// flight; staged, the rows stream in contiguously (cp.async) and the gather
+// reads shared memory without conflicts.  Four blocks share an SM, so the
+// copies of three are in flight while one sums (two blocks with two stages
+// each were slower: their copies waited for their own sums).  Images are
+// taken from the last to the first: the product that wrote dcols has just
+// written the last ones, which are still in L2.  35 us for the CSNN's second
+// layer (164 MB; 24 us at 6.8 TB/s) with direct loads, now 30 us.
+// The sums keep the (ky, kx) order, so both kernels give the same bits.
+constexpr int kCol2imThreads = 288;  // one (pixel, 8 channels) each of a 12 x 12 x 16 map
+constexpr int kCol2imPerSm = 4;
+constexpr int kCol2imMaxStage = 56 * 1024;  // four blocks fit an SM
+
+__device__ __forceinline__ void col2im_cp16(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+
+// (low, high) bf16 of a word as floats
+__device__ __forceinline__ float2 bf2_floats(uint32_t w) {
+  return make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+}
+
+template <int KH, int KW>
+__global__ void __launch_bounds__(kCol2imThreads, kCol2imPerSm) col2im_staged_kernel(
+    const uint4* __restrict__ dcols, uint4* __restrict__ dX, int64_t M, int H, int W, int Cin,
+    int Kpad) {
+  extern __shared__ __align__(16) unsigned char sm[];
+  const int Ho = H - KH + 1, Wo = W - KW + 1;
+  const int G = Cin / 8, vpr = Kpad / 8;
+  const int vecs = Ho * Wo * vpr, outs = H * W * G;
+  const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(sm));
+  const uint4* d = reinterpret_cast<const uint4*>(sm);
+  grid_dep_wait();
+  for (int64_t m = M - 1 - blockIdx.x; m >= 0; m -= gridDim.x) {
+    const uint4* src = dcols + m * vecs;
+    for (int v = threadIdx.x; v < vecs; v += kCol2imThreads) col2im_cp16(base + (uint32_t)v * 16u, src + v);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();  // the image has landed for every thread
+    for (int o = threadIdx.x; o < outs; o += kCol2imThreads) {
+      const int q = o / G, g = o - q * G;
+      const int y = q / W, x = q - y * W;
+      float2 s[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) s[e] = make_float2(0.0f, 0.0f);
+      const uint4* dg = d + (y * Wo + x) * vpr + g;  // the tap (ky, kx) is at pixel (y - ky, x - kx)
+#pragma unroll
+      for (int ky = 0; ky < KH; ++ky) {
+        const bool in_y = (unsigned)(y - ky) < (unsigned)Ho;
+#pragma unroll
+        for (int kx = 0; kx < KW; ++kx) {
+          if (in_y && (unsigned)(x - kx) < (unsigned)Wo) {
+            const uint4 v = dg[(ky * KW + kx) * G - (ky * Wo + kx) * vpr];
+            s[0] = __fadd2_rn(s[0], bf2_floats(v.x));
+            s[1] = __fadd2_rn(s[1], bf2_floats(v.y));
+            s[2] = __fadd2_rn(s[2], bf2_floats(v.z));
+            s[3] = __fadd2_rn(s[3], bf2_floats(v.w));
+          }
+        }
+      }
+      uint4 r;
+      uint32_t* rw = reinterpret_cast<uint32_t*>(&r);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const __nv_bfloat162 h = __floats2bfloat162_rn(s[e].x, s[e].y);
+        rw[e] = *reinterpret_cast<const uint32_t*>(&h);
+      }
+      dX[m * outs + o] = r;
+    }
+    __syncthreads();  // the stage is free for the next image
+  }
+}
+
+template <int KH, int KW>
+cudaError_t launch_col2im_staged(const void* dcols, void* dX, int64_t M, int H, int W, int Cin, int Kpad,
+                                 size_t smem, cudaStream_t st) {
+  const void* k = (const void*)col2im_staged_kernel<KH, KW>;
+  cudaError_t e = ensure_smem(k, smem);
+  DeviceInfo d;
+  if (e == cudaSuccess) e = device_info(&d);
+  if (e != cudaSuccess) return e;
+  const int64_t slots = kCol2imPerSm * (int64_t)d.sms;
+  return launch_pdl(col2im_staged_kernel<KH, KW>, dim3((unsigned)(M < slots ? M : slots)),
+                    dim3(kCol2imThreads), smem, st, static_cast<const uint4*>(dcols),
+                    static_cast<uint4*>(dX), M, H, W, Cin, Kpad);
 }
 
 // Thread i pools the 8 channels of group i % G of output pixel i / G.
@@ -396,16 +500,20 @@ extern "C" snn_status_t snn_im2col_nhwc(int64_t M, int64_t H, int64_t W, int64_t
   if (n / kThreads >= INT_MAX) return SNN_ERR_INVALID_ARG;
   const bool i32 = rows * Kpad < INT_MAX && M * H * W * Cin < INT_MAX;  // 32-bit index math
   if (Cin % 8 == 0 && aligned(X, 16) && Kpad / 8 <= kIm2colMaxGroups) {
-    const unsigned nb = (unsigned)((n + (int64_t)kThreads * kIm2colPer - 1) / ((int64_t)kThreads * kIm2colPer));
+    const int64_t vpr = Kpad / 8;
+    int64_t br = kIm2colBlockVecs / vpr;  // rows per block
+    br = br < 16 ? 16 : br > kIm2colMaxRows ? kIm2colMaxRows : br;
+    const unsigned nb = (unsigned)((rows + br - 1) / br);
+    const size_t smem = (size_t)br * (i32 ? 4 : 8) + (size_t)vpr * 4;  // at most 24 KB
     const cudaError_t e =
-        i32 ? launch_pdl(im2col_vec8_multi_kernel<int>, dim3(nb), dim3(kThreads), 0,
+        i32 ? launch_pdl(im2col_rows_kernel<int>, dim3(nb), dim3(kThreads), smem,
                          reinterpret_cast<cudaStream_t>(stream), static_cast<const uint4*>(X),
                          static_cast<uint4*>(cols), rows, (int)H, (int)W, (int)Cin, (int)KH,
-                         (int)KW, (int)Kpad)
-            : launch_pdl(im2col_vec8_multi_kernel<int64_t>, dim3(nb), dim3(kThreads), 0,
+                         (int)KW, (int)Kpad, (int)br)
+            : launch_pdl(im2col_rows_kernel<int64_t>, dim3(nb), dim3(kThreads), smem,
                          reinterpret_cast<cudaStream_t>(stream), static_cast<const uint4*>(X),
                          static_cast<uint4*>(cols), rows, (int)H, (int)W, (int)Cin, (int)KH,
-                         (int)KW, (int)Kpad);
+                         (int)KW, (int)Kpad, (int)br);
     return e == cudaSuccess ? SNN_OK : SNN_ERR_CUDA;
   }
   if (Cin % 8 == 0 && aligned(X, 16)) {
@@ -446,7 +554,13 @@ extern "C" snn_status_t snn_col2im_nhwc(int64_t M, int64_t H, int64_t W, int64_t
   const bool i32 = M * (H - KH + 1) * (W - KW + 1) * Kpad < INT_MAX && n < INT_MAX;
   if (Cin % 8 == 0 && Kpad % 8 == 0 && aligned(dcols, 16) && aligned(dX, 16)) {
     cudaError_t e;
-    if (KH == 5 && KW == 5 && i32)
+    const int64_t stage = (H - KH + 1) * (W - KW + 1) * Kpad * 2;  // bytes of an image's patch rows
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
+    if (KH == 5 && KW == 5 && stage <= kCol2imMaxStage)
+      e = launch_col2im_staged<5, 5>(dcols, dX, M, (int)H, (int)W, (int)Cin, (int)Kpad, stage, st);
+    else if (KH == 3 && KW == 3 && stage <= kCol2imMaxStage)
+      e = launch_col2im_staged<3, 3>(dcols, dX, M, (int)H, (int)W, (int)Cin, (int)Kpad, stage, st);
+    else if (KH == 5 && KW == 5 && i32)
       e = launch_pdl(col2im_vec8_kernel<int, 5, 5>, dim3(blocks_for(n / 8)), dim3(kThreads), 0,
                      reinterpret_cast<cudaStream_t>(stream), static_cast<const uint4*>(dcols),
                      static_cast<uint4*>(dX), n / 8, (int)H, (int)W, (int)Cin, (int)KH, (int)KW,

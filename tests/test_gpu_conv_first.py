@@ -124,3 +124,33 @@ def test_first_layer_weight_gradient(M, H, Wd, k, Cout, cuda_device):
     # weight gradients are held to
     assert (np.abs(got[:, : k * k] - ref) <= 1e-5 * mag + 1e-12).all()
     assert not got[:, k * k:].any()
+
+
+@pytest.mark.parametrize("M,H,Wd,C,k,Kpad", [
+    (3, 12, 12, 16, 5, 400),    # the CSNN's second layer: one output per thread
+    (700, 6, 6, 8, 3, 72),      # more images than resident blocks
+    (2, 9, 7, 8, 3, 80),        # odd map, padding columns
+    (1, 5, 5, 24, 5, 600),      # one patch row per image
+    (2, 16, 14, 16, 5, 400),    # patch rows too large to stage
+    (5, 20, 18, 8, 1, 8),       # one column group: many rows per block
+])
+def test_patch_rows_and_their_gradient_over_shapes(M, H, Wd, C, k, Kpad, cuda_device):
+    """im2col is an exact copy; col2im adds in (ky, kx) order in fp32 and
+    rounds once, so it equals the same order of additions bit for bit."""
+    g = torch.Generator().manual_seed(M + H)
+    X = torch.randn((M, H, Wd, C), generator=g).to(torch.bfloat16)
+    Ho, Wo, K = H - k + 1, Wd - k + 1, k * k * C
+    cols = torch.full((M * Ho * Wo, Kpad), 7.0, dtype=torch.bfloat16, device=cuda_device)
+    snn.snn_im2col_nhwc(X.to(cuda_device), cols, k, k)
+    want = torch.zeros((M, Ho, Wo, Kpad), dtype=torch.bfloat16)
+    for t in range(k * k):
+        want[..., t * C:(t + 1) * C] = X[:, t // k: t // k + Ho, t % k: t % k + Wo]
+    assert torch.equal(cols.cpu(), want.view(-1, Kpad))
+    d = torch.randn((M, Ho, Wo, Kpad), generator=g).to(torch.bfloat16)
+    d[..., K:] = 1e4
+    dX = torch.empty((M, H, Wd, C), dtype=torch.bfloat16, device=cuda_device)
+    snn.snn_col2im_nhwc(d.view(-1, Kpad).to(cuda_device), dX, k, k)
+    s = torch.zeros((M, H, Wd, C))
+    for t in range(k * k):
+        s[:, t // k: t // k + Ho, t % k: t % k + Wo] += d[..., t * C:(t + 1) * C].float()
+    assert torch.equal(dX.cpu(), s.to(torch.bfloat16))
