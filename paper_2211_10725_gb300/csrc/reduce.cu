@@ -1,5 +1,7 @@
-// Deterministic reduction of per-lane parameter-gradient partials (fp32, one
-// per lane, already summed over t by the scan) into the parameter's shape:
+// Deterministic reduction of parameter-gradient partials (fp32, already summed
+// over t by the scan; one per lane, or, from the staged scans, one per warp,
+// per warp and channel, or per run of a channel's lanes, see PART_* in
+// scan_kernels.cuh) into the parameter's shape:
 // scalar, per neuron [N] (sum over b) or per channel [C] (sum over b and the
 // channel's H*W positions).  Each thread adds its own run of lanes in fp32
 // (tens of terms: an error of a few 1e-6 of their magnitudes), and
@@ -74,6 +76,10 @@ struct ReduceJobs {
 
 // True in every thread of the block that finished a group last.
 __device__ __forceinline__ bool last_of_group(int* ticket, int splits) {
+  if (splits == 1) {  // the group's only block: no ticket to take
+    __syncthreads();  // its partial is visible to the block
+    return true;
+  }
   __shared__ int last;
   __threadfence();  // this block's partial is visible before its ticket
   __syncthreads();
@@ -95,7 +101,8 @@ __global__ void __launch_bounds__(kRedThreads) reduce_scalar(ReduceJobs js, int6
   // a thread's run of lanes (16 at the default chunk) in fp32, in order;
   // everything above compensated
   float acc = 0.0f;
-  for (int64_t l = lo + threadIdx.x; l < hi; l += blockDim.x) acc += j.part[l];
+#pragma unroll 8
+  for (int64_t l = lo + threadIdx.x; l < hi; l += kRedThreads) acc += j.part[l];
   const float2 s = block_sum(make_float2(acc, 0.0f), sh);
   if (threadIdx.x == 0) j.scratch[blockIdx.y] = s;
   if (!last_of_group(&j.tickets[0], S)) return;

@@ -16,23 +16,44 @@ constexpr bool kSpecialise =
     (std::is_same<TI, __nv_bfloat16>::value && std::is_same<TO, __nv_bfloat16>::value) ||
     (std::is_same<TI, float>::value && std::is_same<TO, __nv_bfloat16>::value);
 
-template <bool SYN, typename TI, typename TO, int RESET, bool REC = false>
-cudaError_t fwd_staged(ScanArgs a, cudaStream_t st, bool* launched) {
-  const void* k = (const void*)scan_fwd_staged<SYN, TI, TO, RESET, REC>;
+// Few lanes for the GPU: with 8 lanes a thread, an SM would hold fewer than
+// about 8 warps.
+inline bool few_lanes(int64_t L) {
+  DeviceInfo d;
+  return device_info(&d) == cudaSuccess && L < 2048 * (int64_t)d.sms;
+}
+
+template <bool SYN, typename TI, typename TO, int RESET, bool REC, int VL, bool STRIPS>
+cudaError_t fwd_staged_vl(ScanArgs a, cudaStream_t st, bool* launched) {
+  const void* k = (const void*)scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, STRIPS>;
   StagedPlan p;
   // a stage holds kFwdRows steps of the strip's input row; one CTA per SM
   // where it fits (the longer rows stream faster), two for short sequences
   // (T <= 64: a CTA's few stages fill and drain while the SM's other CTA
   // computes; measured 2-4% faster at T = 25, 0.5% slower at T = 500)
-  if (!plan_staged(k, a.L, ceil_div(a.T, kFwdRows), kFwdRows * (int)sizeof(TI), 0, kLanes<SYN>, &p,
-                   0, 0, a.T <= 64 ? 2 : 1))
+  if (!plan_staged(k, a.L, ceil_div(a.T, kFwdRows), kFwdRows * (int)sizeof(TI), 0, VL, &p, 0, 0,
+                   a.T <= 64 ? 2 : 1))
     return cudaSuccess;
   a.lanes_per_cta = p.lanes_per_cta;
   a.stages = p.stages;
   a.stage_bytes = p.stage_bytes;
   *launched = true;
-  return launch_pdl(scan_fwd_staged<SYN, TI, TO, RESET, REC>, dim3((unsigned)p.grid),
+  const int64_t grid = STRIPS && p.resident < p.grid ? p.resident : p.grid;
+  return launch_pdl(scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, STRIPS>, dim3((unsigned)grid),
                     dim3(p.threads), p.smem, st, a);
+}
+
+// Short sequences (T <= 64) take 4 lanes a thread and CTAs that walk their
+// strips: with one CTA per strip each wave paid the ring's fill and drain
+// (T = 25, 128 x 6912 lanes in fp32, both passes: 127 us with 8 lanes and
+// three waves, 98 us so; 78 us at 6.8 TB/s).  Longer ones take 8 lanes
+// (Leaky; T = 500, 64 x 8192 lanes: 9% faster than 4 in store mode) unless
+// the lanes are few (T = 100, 64 x 4096: 20% slower than 4).
+template <bool SYN, typename TI, typename TO, int RESET, bool REC = false>
+cudaError_t fwd_staged(ScanArgs a, cudaStream_t st, bool* launched) {
+  if (a.T <= 64) return fwd_staged_vl<SYN, TI, TO, RESET, REC, 4, true>(a, st, launched);
+  if (!SYN && few_lanes(a.L)) return fwd_staged_vl<SYN, TI, TO, RESET, REC, 4, false>(a, st, launched);
+  return fwd_staged_vl<SYN, TI, TO, RESET, REC, kLanes<SYN>, false>(a, st, launched);
 }
 
 template <bool SYN, typename TI, typename TO>
@@ -66,13 +87,14 @@ cudaError_t bwd_staged_vl(ScanArgs a, cudaStream_t st, bool* launched) {
     items = 2 * a.T;
   } else {
     const int n = 2 + (sizeof(TO) != 4 ? 1 : 0) + ((SYN && a.part_alpha) ? 1 : 0) + (a.gm ? 1 : 0);
-    per_lane = n * (int)sizeof(TO);
+    per_lane = kBwdRows * n * (int)sizeof(TO);
     seg = 0;
     fixed = 0;
-    items = a.T;
+    items = ceil_div(a.T, kBwdRows);
   }
   StagedPlan p;
-  if (!plan_staged(k, a.L, items, per_lane, seg, VL, &p, fixed, KC)) return cudaSuccess;
+  if (!plan_staged(k, a.L, items, per_lane, seg, VL, &p, fixed, KC, 2, part_align(a))) return cudaSuccess;
+  choose_parts(a, p, VL);
   a.lanes_per_cta = p.lanes_per_cta;
   a.stages = p.stages;
   a.stage_bytes = p.stage_bytes;
@@ -82,12 +104,13 @@ cudaError_t bwd_staged_vl(ScanArgs a, cudaStream_t st, bool* launched) {
 }
 
 // The staged backward with its lanes per thread: 4 for the Leaky neuron's
-// store mode on sequences of at most 64 steps, else kLanes.
+// store mode on sequences of at most 64 steps or with few lanes, else kLanes.
 template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int KC = 0,
           bool REC = false>
 cudaError_t bwd_staged(ScanArgs a, cudaStream_t st, bool* launched) {
   if constexpr (!SYN && !RECOMP) {
-    if (a.T <= 64) return bwd_staged_vl<SYN, RECOMP, TI, TO, RESET, SG, KC, REC, 4>(a, st, launched);
+    if (a.T <= 64 || few_lanes(a.L))
+      return bwd_staged_vl<SYN, RECOMP, TI, TO, RESET, SG, KC, REC, 4>(a, st, launched);
   }
   return bwd_staged_vl<SYN, RECOMP, TI, TO, RESET, SG, KC, REC, kLanes<SYN>>(a, st, launched);
 }

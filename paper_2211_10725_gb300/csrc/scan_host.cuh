@@ -64,7 +64,8 @@ struct StagedPlan {
   int stages = 0;
   int stage_bytes = 0;
   size_t smem = 0;
-  int64_t grid = 0;
+  int64_t grid = 0;      // strips
+  int64_t resident = 0;  // CTAs that run at once
 };
 
 // Choose a staged launch for L lanes: all CTAs of a wave resident at once
@@ -77,16 +78,18 @@ struct StagedPlan {
 //   fixed_bytes_per_lane: other shared memory per lane of the strip
 //   force_stages: exact ring depth the kernel was compiled for (0 = any)
 //   max_cps: most CTAs per SM to try (larger strips first when 1)
+//   lane_align: the strips' lanes are a multiple of it (8, 16 or 32)
 inline bool plan_staged(const void* kernel, int64_t L, int64_t items, int stage_bytes_per_lane,
                         int seg_bytes_per_thread, int lanes_per_thread, StagedPlan* plan,
-                        int fixed_bytes_per_lane = 0, int force_stages = 0, int max_cps = 2) {
+                        int fixed_bytes_per_lane = 0, int force_stages = 0, int max_cps = 2,
+                        int lane_align = 8) {
   static std::mutex mu;
-  static std::map<std::tuple<int, const void*, int64_t, int64_t, int, int>, StagedPlan> cache;
+  static std::map<std::tuple<int, const void*, int64_t, int64_t, int, int, int>, StagedPlan> cache;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   const auto key = std::make_tuple(dev, kernel, L, items, stage_bytes_per_lane,
                                    ((seg_bytes_per_thread * 64 + fixed_bytes_per_lane) * 64 +
-                                    force_stages) * 4 + max_cps);
+                                    force_stages) * 4 + max_cps, lane_align);
   {
     std::lock_guard<std::mutex> g(mu);
     auto it = cache.find(key);
@@ -103,7 +106,7 @@ inline bool plan_staged(const void* kernel, int64_t L, int64_t items, int stage_
   for (int waves = 1; waves <= 64; ++waves) {
     for (int cps = max_cps; cps >= 1; --cps) {
       const int64_t ctas = (int64_t)d.sms * cps * waves;
-      const int64_t lpc = round_up(ceil_div(L, ctas), 8);
+      const int64_t lpc = round_up(ceil_div(L, ctas), lane_align);
       const int64_t cthreads = round_up(ceil_div(lpc, lanes_per_thread), 32);
       const int threads = (int)cthreads + 32;
       if (threads > kMaxStagedThreads) continue;
@@ -125,6 +128,7 @@ inline bool plan_staged(const void* kernel, int64_t L, int64_t items, int stage_
       p.stage_bytes = (int)stage_bytes;
       p.smem = (size_t)(kBarrierBytes + stages * stage_bytes + seg_bytes);
       p.grid = ceil_div(L, lpc);
+      p.resident = (int64_t)d.sms * cps;
       if (ensure_smem(kernel, p.smem) != cudaSuccess) continue;
       int nb = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, p.smem) != cudaSuccess)
@@ -137,6 +141,48 @@ inline bool plan_staged(const void* kernel, int64_t L, int64_t items, int stage_
     }
   }
   return false;
+}
+
+// Lane alignment of the strips for the partials of a per-channel parameter
+// with HW > 1 positions per channel: runs of up to 32 lanes of one channel
+// then lie within one warp (32 rather than more: a strip of a small layer
+// stays near its even share of the lanes).
+inline int part_align(const ScanArgs& a) {
+  const bool chan = (a.part_beta && a.beta_mode == PM_PER_CHANNEL) ||
+                    (a.part_thr && a.thr_mode == PM_PER_CHANNEL) ||
+                    (a.part_alpha && a.alpha_mode == PM_PER_CHANNEL);
+  if (!chan || a.HW < 16 || a.N % a.HW != 0) return VEC;
+  return a.HW % 32 == 0 ? 32 : a.HW % 16 == 0 ? 16 : VEC;
+}
+
+// Layout of each parameter's partials for a staged launch with `lanes` lanes
+// per thread (see PART_*); the caller's reduction reads it from part_info.
+// PART_CHANNELS only where the warps' channel rows are fewer than the lanes
+// (a strip of a few lanes would write more than one float per lane, and
+// past the workspace).
+inline void choose_parts(ScanArgs& a, const StagedPlan& p, int lanes) {
+  const int64_t warps = p.grid * (p.threads / 32 - 1);
+  const float* part[3] = {a.part_beta, a.part_thr, a.part_alpha};
+  const int mode[3] = {a.beta_mode, a.thr_mode, a.alpha_mode};
+  int q = part_align(a);
+  if (p.lanes_per_cta % q != 0 || a.HW % q != 0) q = 0;
+  for (int k = 0; k < 3; ++k) {
+    int kind = PART_LANE;
+    if (part[k] && mode[k] == PM_SCALAR) {
+      kind = PART_WARP;
+    } else if (part[k] && mode[k] == PM_PER_CHANNEL) {
+      const bool pow2 = (a.C & (a.C - 1)) == 0;
+      if (a.HW == 1 && pow2 && a.C >= lanes && a.C <= 16 * lanes && warps * a.C <= a.L) kind = PART_CHANNELS;
+      else if (a.HW > 1 && q >= lanes) kind = PART_RUN;
+    }
+    a.part_kind[k] = kind;
+    if (a.part_info) a.part_info->kind[k] = kind;
+  }
+  a.part_q = q;
+  if (a.part_info) {
+    a.part_info->warps = warps;
+    a.part_info->q = q;
+  }
 }
 
 // Entry points of the per-translation-unit dispatchers.  dtype codes follow

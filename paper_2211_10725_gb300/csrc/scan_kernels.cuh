@@ -38,6 +38,23 @@ constexpr int kMaxStages = 60;
 constexpr int kMaxStagedThreads = 512;
 constexpr uint64_t kDrainNs = 1000000000ull;
 
+// Layouts of a parameter's gradient partials in the workspace.  The staged
+// kernels add the partials of a warp that belong to one value of the
+// parameter before they leave the chip, so the reduction that follows reads
+// a fraction of one float per lane.
+enum {
+  PART_LANE = 0,     // one per lane
+  PART_WARP = 1,     // scalar: one per consumer warp
+  PART_CHANNELS = 2, // per channel, HW = 1, C a power of two: C per consumer warp
+  PART_RUN = 3       // per channel, HW > 1: one per part_q neighbouring lanes (part_q divides HW)
+};
+// What a launch wrote, for the reduction (host memory).
+struct PartInfo {
+  int kind[3];    // of beta, thr, alpha
+  int64_t warps;  // consumer warps of the launch
+  int q;          // lanes per PART_RUN partial
+};
+
 struct ScanArgs {
   int64_t T, L, N, C, HW;
   int K;      // checkpoint interval (recompute); T in store mode
@@ -75,6 +92,9 @@ struct ScanArgs {
   float* part_beta;  // per-lane parameter-gradient partials (workspace) or null
   float* part_thr;
   float* part_alpha;
+  int part_kind[3];    // layout of each (PART_*)
+  int part_q;          // lanes per PART_RUN partial
+  PartInfo* part_info; // host: set by the launcher
   float* gmem0;
   float* gsyn0;
   // control
@@ -546,6 +566,39 @@ __device__ __forceinline__ void initial_state(const ScanArgs& a, int64_t l, cons
   }
 }
 
+// One parameter's gradient partials of a consumer warp, in the layout the
+// launch chose; every lane of the warp calls it (an inactive thread adds
+// zeros).  gw: the warp's index among the launch's consumer warps.
+template <int V>
+__device__ __forceinline__ void store_partials(const ScanArgs& a, float* part, int kind, float (&v)[V],
+                                               int64_t l, bool active, int64_t gw, int lid) {
+  if (kind == PART_LANE) {
+    if (active) storev<float, V>(part + l, v);
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < V; ++k)
+    if (!active) v[k] = 0.0f;
+  if (kind == PART_CHANNELS) {  // threads C / V apart hold the same channels
+    const int period = (int)a.C / V;
+    for (int d = period; d < 32; d <<= 1)
+#pragma unroll
+      for (int k = 0; k < V; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], d);
+    if (lid < period) storev<float, V>(part + gw * a.C + (l & (a.C - 1)), v);
+    return;
+  }
+  float s = 0.0f;
+#pragma unroll
+  for (int k = 0; k < V; k += 2) s += v[k] + v[k + 1];
+  const int group = kind == PART_WARP ? 32 : a.part_q / V;  // threads that add up
+  for (int d = 1; d < group; d <<= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+  if (kind == PART_WARP) {
+    if (lid == 0) part[gw] = s;
+  } else if (active && (lid & (group - 1)) == 0) {
+    part[l / a.part_q] = s;
+  }
+}
+
 // ---------------------------------------------------------------------------
 // Staged forward
 // ---------------------------------------------------------------------------
@@ -554,9 +607,14 @@ __device__ __forceinline__ void initial_state(const ScanArgs& a, int64_t l, cons
 // release per kFwdRows steps instead of per step.
 constexpr int kFwdRows = 8;
 
-template <bool SYN, typename TI, typename TO, int RESET, bool REC = false>
+// VL: lanes per thread.  STRIPS: a CTA walks the strips blockIdx.x, blockIdx.x
+// + gridDim.x, ... (else the grid has one CTA per strip): the ring runs on
+// across strips, so the next strip's rows arrive while the last steps of the
+// current one are computed.
+template <bool SYN, typename TI, typename TO, int RESET, bool REC = false, int VL = kLanes<SYN>,
+          bool STRIPS = false>
 __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanArgs a) {
-  constexpr int V = kLanes<SYN>, NP = V / 2, R = kFwdRows;
+  constexpr int V = VL, NP = V / 2, R = kFwdRows;
   extern __shared__ __align__(1024) unsigned char smem[];
   uint64_t* full = reinterpret_cast<uint64_t*>(smem);
   uint64_t* empty = full + kMaxStages;
@@ -564,8 +622,6 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanA
   const int S = a.stages;
   const int cwarps = (int)(blockDim.x >> 5) - 1;
   const int warp = threadIdx.x >> 5, lid = threadIdx.x & 31;
-  const int64_t lane0 = (int64_t)blockIdx.x * a.lanes_per_cta;
-  const int cta_lanes = (int)min((int64_t)a.lanes_per_cta, a.L - lane0);
   const int row_elems = a.lanes_per_cta;  // a stage holds R rows of the strip
   init_ring_barriers(full, empty, S, cwarps);
   grid_dep_wait();  // the previous kernel on the stream is complete
@@ -573,14 +629,19 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanA
   if (warp == cwarps) {  // producer warp
     if (lid == 0 && !(a.debug & DEBUG_PRODUCER_IDLE)) {
       Producer p{ring, full, empty, S, a.stage_bytes};
-      const uint32_t bytes = (uint32_t)cta_lanes * (uint32_t)sizeof(TI);
       const uint32_t row_bytes = (uint32_t)row_elems * (uint32_t)sizeof(TI);
-      const TI* src = static_cast<const TI*>(a.I) + lane0;
-      for (int64_t t0 = 0; t0 < a.T; t0 += R) {
-        const int nr = (int)min((int64_t)R, a.T - t0);
-        if (!p.begin((uint32_t)nr * bytes, a)) break;
-        for (int r = 0; r < nr; ++r) p.copy((uint32_t)r * row_bytes, src + (t0 + r) * a.L, bytes);
-        p.end();
+      for (int64_t lane0 = (int64_t)blockIdx.x * a.lanes_per_cta; lane0 < a.L && p.ok;
+           lane0 += (int64_t)gridDim.x * a.lanes_per_cta) {
+        const int cta_lanes = (int)min((int64_t)a.lanes_per_cta, a.L - lane0);
+        const uint32_t bytes = (uint32_t)cta_lanes * (uint32_t)sizeof(TI);
+        const TI* src = static_cast<const TI*>(a.I) + lane0;
+        for (int64_t t0 = 0; t0 < a.T; t0 += R) {
+          const int nr = (int)min((int64_t)R, a.T - t0);
+          if (!p.begin((uint32_t)nr * bytes, a)) break;
+          for (int r = 0; r < nr; ++r) p.copy((uint32_t)r * row_bytes, src + (t0 + r) * a.L, bytes);
+          p.end();
+        }
+        if (!STRIPS) break;
       }
       p.drain();
     }
@@ -588,100 +649,109 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanA
   }
 
   const int c = threadIdx.x;
-  const int64_t l = lane0 + (int64_t)c * V;
-  const bool active = c * V < cta_lanes;
-  float2 beta[NP], negthr[NP], third[NP], u[NP], z[NP], in[NP];
-  if (active) {
-    load_params<SYN || REC, NP>(a, l, beta, negthr, third);
-    bool zb[V];
-    initial_state<SYN, NP>(a, l, negthr, u, zb, in);
-#pragma unroll
-    for (int k = 0; k < NP; ++k) {
-      z[k] = make_float2(zb[2 * k] ? 1.0f : 0.0f, zb[2 * k + 1] ? 1.0f : 0.0f);
-      if (REC) third[k] = add2_rn(third[k], negthr[k]);  // v - thr, rounded once
-    }
-  }
-  TO* spk = static_cast<TO*>(a.spk) + l;
-  TO* mem = a.mem ? static_cast<TO*>(a.mem) + l : nullptr;
-  TO* syn = (SYN && a.syn) ? static_cast<TO*>(a.syn) + l : nullptr;
-  float* ck = a.ckpt ? a.ckpt + l : nullptr;
-  const int64_t ck_stride = SYN ? 2 * a.L : a.L;
-  // spike bits: one byte per thread and step (Leaky, 8 lanes), or one per
-  // pair of threads (Synaptic, 4 lanes each: the even thread stores)
-  unsigned char* bits = a.bits ? a.bits + lane0 / 8 + (SYN ? c / 2 : c) : nullptr;
   const TI* my = reinterpret_cast<const TI*>(ring) + c * V;
   const int stage_elems = a.stage_bytes / (int)sizeof(TI);
   RingPos pos;
-  int kk = a.nseg > 0 ? seg_phase0(a) : 0;  // position inside the current checkpoint segment
-  for (int64_t t0 = 0; t0 < a.T; t0 += R) {
-    if (!warp_wait(&full[pos.s], pos.ph, a.wait_ns)) {
-      if (lid == 0) record_status(a.status, kStatusTimeout);
-      break;
-    }
-    const int nr = (int)min((int64_t)R, a.T - t0);
-    unsigned zbits[R];
+  for (int64_t lane0 = (int64_t)blockIdx.x * a.lanes_per_cta; lane0 < a.L;
+       lane0 += (int64_t)gridDim.x * a.lanes_per_cta) {
+    const int cta_lanes = (int)min((int64_t)a.lanes_per_cta, a.L - lane0);
+    const int64_t l = lane0 + (int64_t)c * V;
+    const bool active = c * V < cta_lanes;
+    float2 beta[NP], negthr[NP], third[NP], u[NP], z[NP], in[NP];
     if (active) {
-      const TI* st = my + pos.s * stage_elems;
+      load_params<SYN || REC, NP>(a, l, beta, negthr, third);
+      bool zb[V];
+      initial_state<SYN, NP>(a, l, negthr, u, zb, in);
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        zbits[r] = 0;
-        if (r < nr) {
-          float2 x[NP];
-          load_pairs<TI, NP>(st + r * row_elems, x);
+      for (int k = 0; k < NP; ++k) {
+        z[k] = make_float2(zb[2 * k] ? 1.0f : 0.0f, zb[2 * k + 1] ? 1.0f : 0.0f);
+        if (REC) third[k] = add2_rn(third[k], negthr[k]);  // v - thr, rounded once
+      }
+    }
+    TO* spk = static_cast<TO*>(a.spk) + l;
+    TO* mem = a.mem ? static_cast<TO*>(a.mem) + l : nullptr;
+    TO* syn = (SYN && a.syn) ? static_cast<TO*>(a.syn) + l : nullptr;
+    float* ck = a.ckpt ? a.ckpt + l : nullptr;
+    const int64_t ck_stride = SYN ? 2 * a.L : a.L;
+    // spike bits: one byte per thread and step (8 lanes), or one per pair of
+    // threads (4 lanes each: the even thread stores)
+    unsigned char* bits = a.bits ? a.bits + lane0 / 8 + (V == 4 ? c / 2 : c) : nullptr;
+    int kk = a.nseg > 0 ? seg_phase0(a) : 0;  // position inside the current checkpoint segment
+    for (int64_t t0 = 0; t0 < a.T; t0 += R) {
+      if (!warp_wait(&full[pos.s], pos.ph, a.wait_ns)) {
+        if (lid == 0) record_status(a.status, kStatusTimeout);
+        return;
+      }
+      const int nr = (int)min((int64_t)R, a.T - t0);
+      unsigned zbits[R];
+      if (active) {
+        const TI* st = my + pos.s * stage_elems;
 #pragma unroll
-          for (int k = 0; k < NP; ++k)
-            fwd_pair<SYN, RESET, REC ? 1 : 0>(a.reset, beta[k], negthr[k], third[k], x[k], u[k],
-                                              z[k], in[k]);
-          if (bits) {
+        for (int r = 0; r < R; ++r) {
+          zbits[r] = 0;
+          if (r < nr) {
+            float2 x[NP];
+            load_pairs<TI, NP>(st + r * row_elems, x);
 #pragma unroll
-            for (int k = 0; k < NP; ++k) {
-              zbits[r] |= ((z[k].x != 0.0f) ? 1u : 0u) << (2 * k);
-              zbits[r] |= ((z[k].y != 0.0f) ? 1u : 0u) << (2 * k + 1);
+            for (int k = 0; k < NP; ++k)
+              fwd_pair<SYN, RESET, REC ? 1 : 0>(a.reset, beta[k], negthr[k], third[k], x[k], u[k],
+                                                z[k], in[k]);
+            if (bits) {
+#pragma unroll
+              for (int k = 0; k < NP; ++k) {
+                zbits[r] |= ((z[k].x != 0.0f) ? 1u : 0u) << (2 * k);
+                zbits[r] |= ((z[k].y != 0.0f) ? 1u : 0u) << (2 * k + 1);
+              }
             }
-          }
-          store_pairs<TO, NP>(spk + r * a.L, z);
-          if (mem) store_pairs<TO, NP>(mem + r * a.L, u);
-          if (SYN && syn) store_pairs<TO, NP>(syn + r * a.L, in);
-          if (++kk == a.K) {
-            kk = 0;
-            if (ck && t0 + r + 1 < a.T) {
-              store_pairs<float, NP>(ck, u);
-              if (SYN) store_pairs<float, NP>(ck + a.L, in);
-              ck += ck_stride;
+            store_pairs<TO, NP>(spk + r * a.L, z);
+            if (mem) store_pairs<TO, NP>(mem + r * a.L, u);
+            if (SYN && syn) store_pairs<TO, NP>(syn + r * a.L, in);
+            if (++kk == a.K) {
+              kk = 0;
+              if (ck && t0 + r + 1 < a.T) {
+                store_pairs<float, NP>(ck, u);
+                if (SYN) store_pairs<float, NP>(ck + a.L, in);
+                ck += ck_stride;
+              }
             }
           }
         }
       }
-    }
-    if (bits) {
+      if (bits) {
 #pragma unroll
-      for (int r = 0; r < R; ++r) {
-        if (r < nr) {
-          if (SYN) {
-            const unsigned hi = __shfl_down_sync(0xffffffffu, zbits[r], 1);
-            if (active && !(c & 1)) bits[r * a.bits_row] = (unsigned char)(zbits[r] | (hi << 4));
-          } else if (active) {
-            bits[r * a.bits_row] = (unsigned char)zbits[r];
+        for (int r = 0; r < R; ++r) {
+          if (r < nr) {
+            if (V == 4) {
+              const unsigned hi = __shfl_down_sync(0xffffffffu, zbits[r], 1);
+              if (active && !(c & 1)) bits[r * a.bits_row] = (unsigned char)(zbits[r] | (hi << 4));
+            } else if (active) {
+              bits[r * a.bits_row] = (unsigned char)zbits[r];
+            }
           }
         }
+        bits += R * a.bits_row;
       }
-      bits += R * a.bits_row;
+      release_stage(empty, pos.s, lid);
+      pos.next(S);
+      spk += R * a.L;
+      if (mem) mem += R * a.L;
+      if (SYN && syn) syn += R * a.L;
     }
-    release_stage(empty, pos.s, lid);
-    pos.next(S);
-    spk += R * a.L;
-    if (mem) mem += R * a.L;
-    if (SYN && syn) syn += R * a.L;
-  }
-  if (active) {
-    if (a.mem_final) store_pairs<float, NP>(a.mem_final + l, u);
-    if (SYN && a.syn_final) store_pairs<float, NP>(a.syn_final + l, in);
+    if (active) {
+      if (a.mem_final) store_pairs<float, NP>(a.mem_final + l, u);
+      if (SYN && a.syn_final) store_pairs<float, NP>(a.syn_final + l, in);
+    }
+    if (!STRIPS) break;
   }
 }
 
 // ---------------------------------------------------------------------------
-// Staged backward.  Store mode (RECOMP=false): one item per step t = T-1..0
-// holding the rows {grad_spk, mem, [spk], [syn], [grad_mem]}.  Recompute
+// Staged backward.  Store mode (RECOMP=false): one item per kBwdRows steps,
+// from t = T-1 down, holding for each of them the rows {grad_spk, mem, [spk],
+// [syn], [grad_mem]} (with one step per item the barriers' rate, not the
+// bytes in flight, bounded the half-precision scans: with 4, and 4 lanes a
+// thread, the recurrent neuron's two passes at T = 100 over 64 x 4096 lanes
+// in bf16 went from 90 to 72 us; 46 us at 6.8 TB/s).  Recompute
 // mode: checkpoint segments from last to first; per segment, items for
 // t = t0..t1-1 holding {I, [ckpt u, ckpt i at t0]} replay the forward into a
 // per-thread shared-memory buffer, then items t = t1-1..t0 holding
@@ -703,6 +773,8 @@ __device__ __forceinline__ void bwd_pairs(const ScanArgs& a, const float2 beta[N
                                                   z[2 * k], z[2 * k + 1], i[k], g[k], eu[k],
                                                   ei[k], st[k]);
 }
+
+constexpr int kBwdRows = 4;  // steps per item of the store-mode backward
 
 template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int KC = 0,
           bool REC = false, int VL = kLanes<SYN>>
@@ -729,6 +801,7 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_bwd_staged(const ScanA
   // store-mode tile order: gs, mem, [spk], [syn], [gm]
   const int t_spk = 2, t_syn = 2 + (half_store ? 1 : 0);
   const int t_gm_store = t_syn + ((!RECOMP && want_syn) ? 1 : 0);
+  const int step_tiles = t_gm_store + (a.gm ? 1 : 0);  // tiles of one step of an item
   // recompute: two checkpoint slots after the replay buffer, prefetched one
   // segment ahead (each holds the strip's u row, then its i row)
   uint64_t* ck_full = full + 2 * kMaxStages;
@@ -749,17 +822,21 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_bwd_staged(const ScanA
         const uint32_t nb = (uint32_t)(bits_skew + cta_lanes / 8 + 15) & ~15u;  // bit row
         const int n_io = 2 + ((half_store && !use_bits) ? 1 : 0) + (want_syn ? 1 : 0) + (a.gm ? 1 : 0);
         const uint32_t total = (uint32_t)n_io * bo + (use_bits ? nb : 0u);
-        for (int64_t t = a.T - 1; t >= 0; --t) {
-          if (!p.begin(total, a)) break;
-          uint32_t n = 0;
-          p.copy(n++ * io_stride, row<TO>(a.gs, t, a.L, lane0), bo);
-          p.copy(n++ * io_stride, row<TO>(a.mem_in, t, a.L, lane0), bo);
-          if (use_bits)
-            p.copy(n++ * io_stride, a.bits + t * a.bits_row + lane0 / 8 - bits_skew, nb);
-          else if (half_store)
-            p.copy(n++ * io_stride, row<TO>(a.spk_in, t, a.L, lane0), bo);
-          if (want_syn) p.copy(n++ * io_stride, row<TO>(a.syn_in, t, a.L, lane0), bo);
-          if (a.gm) p.copy(n++ * io_stride, row<TO>(a.gm, t, a.L, lane0), bo);
+        for (int64_t t1 = a.T - 1; t1 >= 0; t1 -= kBwdRows) {
+          const int nr = (int)min((int64_t)kBwdRows, t1 + 1);
+          if (!p.begin((uint32_t)nr * total, a)) break;
+          for (int r = 0; r < nr; ++r) {
+            const int64_t t = t1 - r;
+            uint32_t n = (uint32_t)(r * step_tiles);
+            p.copy(n++ * io_stride, row<TO>(a.gs, t, a.L, lane0), bo);
+            p.copy(n++ * io_stride, row<TO>(a.mem_in, t, a.L, lane0), bo);
+            if (use_bits)
+              p.copy(n++ * io_stride, a.bits + t * a.bits_row + lane0 / 8 - bits_skew, nb);
+            else if (half_store)
+              p.copy(n++ * io_stride, row<TO>(a.spk_in, t, a.L, lane0), bo);
+            if (want_syn) p.copy(n++ * io_stride, row<TO>(a.syn_in, t, a.L, lane0), bo);
+            if (a.gm) p.copy(n++ * io_stride, row<TO>(a.gm, t, a.L, lane0), bo);
+          }
           p.end();
         }
       } else {
@@ -854,52 +931,72 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_bwd_staged(const ScanA
   };
 
   if (!RECOMP) {
-    for (int64_t t = a.T - 1; t >= 0; --t) {
+    // the final state's gradients enter at t = T-1 and are zero below it
+    float2 eu[NP], ei[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) eu[k] = ei[k] = f2(0.0f);
+    if (active && a.gmf) load_pairs_global<NP>(a.gmf + l, eu);
+    if (SYN && active && a.gsf) load_pairs_global<NP>(a.gsf + l, ei);
+    for (int64_t t1 = a.T - 1; t1 >= 0; t1 -= kBwdRows) {
       if (!warp_wait(&full[pos.s], pos.ph, a.wait_ns)) {
         if (lid == 0) record_status(a.status, kStatusTimeout);
         ok = false;
         break;
       }
+      const int nr = (int)min((int64_t)kBwdRows, t1 + 1);
       if (active) {
         const TO* base = ring_o + pos.s * stage_io_elems;
-        float2 g[NP], uu[NP], ii[NP], gmv[NP], out[NP];
-        bool zz[V];
-        load_pairs<TO, NP>(base, g);
-        load_pairs<TO, NP>(base + tile_io_elems, uu);
-        if (use_bits) {
-          const unsigned char* bb = reinterpret_cast<const unsigned char*>(base - c * V) +
-                                    t_spk * io_stride + bits_skew + (V == 4 ? c / 2 : c);
-          const unsigned zb = V == 4 ? (unsigned)(*bb >> ((c & 1) * 4)) : (unsigned)*bb;
 #pragma unroll
-          for (int k = 0; k < V; ++k) zz[k] = (zb >> k) & 1u;
-        } else if (half_store) {
-          float2 sp[NP];
-          load_pairs<TO, NP>(base + t_spk * tile_io_elems, sp);
+        for (int r = 0; r < kBwdRows; ++r) {
+          if (r < nr) {
+            float2 g[NP], uu[NP], ii[NP], gmv[NP], out[NP];
+            bool zz[V];
+            load_pairs<TO, NP>(base, g);
+            load_pairs<TO, NP>(base + tile_io_elems, uu);
+            if (use_bits) {
+              const unsigned char* bb = reinterpret_cast<const unsigned char*>(base - c * V) +
+                                        t_spk * io_stride + bits_skew + (V == 4 ? c / 2 : c);
+              const unsigned zb = V == 4 ? (unsigned)(*bb >> ((c & 1) * 4)) : (unsigned)*bb;
 #pragma unroll
-          for (int k = 0; k < NP; ++k) {
-            zz[2 * k] = sp[k].x != 0.0f;
-            zz[2 * k + 1] = sp[k].y != 0.0f;
-          }
-        } else {
+              for (int k = 0; k < V; ++k) zz[k] = (zb >> k) & 1u;
+            } else if (half_store) {
+              float2 sp[NP];
+              load_pairs<TO, NP>(base + t_spk * tile_io_elems, sp);
 #pragma unroll
-          for (int k = 0; k < NP; ++k) {
-            zz[2 * k] = uu[k].x > -negthr[k].x;
-            zz[2 * k + 1] = uu[k].y > -negthr[k].y;
+              for (int k = 0; k < NP; ++k) {
+                zz[2 * k] = sp[k].x != 0.0f;
+                zz[2 * k + 1] = sp[k].y != 0.0f;
+              }
+            } else {
+#pragma unroll
+              for (int k = 0; k < NP; ++k) {
+                zz[2 * k] = uu[k].x > -negthr[k].x;
+                zz[2 * k + 1] = uu[k].y > -negthr[k].y;
+              }
+            }
+            if (want_syn) {
+              load_pairs<TO, NP>(base + t_syn * tile_io_elems, ii);
+            } else {
+#pragma unroll
+              for (int k = 0; k < NP; ++k) ii[k] = f2(0.0f);
+            }
+            if (a.gm) {
+              load_pairs<TO, NP>(base + t_gm_store * tile_io_elems, gmv);
+#pragma unroll
+              for (int k = 0; k < NP; ++k) eu[k] = add2(eu[k], gmv[k]);
+            }
+            bwd_pairs<SYN, RESET, SG, true, NP, REC>(a, beta, negthr, alpha, uu, zz, ii, g, eu, ei,
+                                                     st, out);
+#pragma unroll
+            for (int k = 0; k < NP; ++k) eu[k] = ei[k] = f2(0.0f);
+            store_pairs<TO, NP>(gI, out);
+            gI -= a.L;
+            base += step_tiles * tile_io_elems;
           }
         }
-        if (want_syn) {
-          load_pairs<TO, NP>(base + t_syn * tile_io_elems, ii);
-        } else {
-#pragma unroll
-          for (int k = 0; k < NP; ++k) ii[k] = f2(0.0f);
-        }
-        if (a.gm) load_pairs<TO, NP>(base + t_gm_store * tile_io_elems, gmv);
-        reverse(t, uu, zz, ii, g, gmv, out);
-        store_pairs<TO, NP>(gI, out);
       }
       release_stage(empty, pos.s, lid);
       pos.next(S);
-      gI -= a.L;
     }
   } else {
     int64_t ck_u = 0;  // checkpoints consumed
@@ -1067,7 +1164,7 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_bwd_staged(const ScanA
       }
     }
   }
-  if (!ok || !active) return;
+  if (!ok) return;
   float gm0[V], gs0[V], db[V], dt[V], da[V];
 #pragma unroll
   for (int v = 0; v < V; ++v) {
@@ -1079,22 +1176,24 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_bwd_staged(const ScanA
     const float th = -(hi ? negthr[v / 2].y : negthr[v / 2].x);
     const float al = hi ? alpha[v / 2].y : alpha[v / 2].x;
     if (a.T == 0) {
-      gm0[v] = a.gmf ? a.gmf[l + v] : 0.0f;
-      gs0[v] = (SYN && a.gsf) ? a.gsf[l + v] : 0.0f;
+      gm0[v] = (active && a.gmf) ? a.gmf[l + v] : 0.0f;
+      gs0[v] = (SYN && active && a.gsf) ? a.gsf[l + v] : 0.0f;
     } else {
-      const float m0 = a.mem0 ? a.mem0[l + v] : 0.0f;
-      const float s0 = (SYN && a.syn0) ? a.syn0[l + v] : 0.0f;
+      const float m0 = (active && a.mem0) ? a.mem0[l + v] : 0.0f;
+      const float s0 = (SYN && active && a.syn0) ? a.syn0[l + v] : 0.0f;
       bwd_initial<SYN>(a, b, th, al, a.mem0 != nullptr, m0, s0, sl, gm0[v], gs0[v]);
     }
     db[v] = sl.dbeta;
     dt[v] = sl.dthr;
     da[v] = sl.dalpha;
   }
-  if (a.gmem0) storev<float, V>(a.gmem0 + l, gm0);
-  if (SYN && a.gsyn0) storev<float, V>(a.gsyn0 + l, gs0);
-  if (a.part_beta) storev<float, V>(a.part_beta + l, db);
-  if (a.part_thr) storev<float, V>(a.part_thr + l, dt);
-  if ((SYN || REC) && a.part_alpha) storev<float, V>(a.part_alpha + l, da);
+  if (active && a.gmem0) storev<float, V>(a.gmem0 + l, gm0);
+  if (SYN && active && a.gsyn0) storev<float, V>(a.gsyn0 + l, gs0);
+  const int64_t gw = (int64_t)blockIdx.x * cwarps + warp;
+  if (a.part_beta) store_partials<V>(a, a.part_beta, a.part_kind[0], db, l, active, gw, lid);
+  if (a.part_thr) store_partials<V>(a, a.part_thr, a.part_kind[1], dt, l, active, gw, lid);
+  if ((SYN || REC) && a.part_alpha)
+    store_partials<V>(a, a.part_alpha, a.part_kind[2], da, l, active, gw, lid);
 }
 
 // ---------------------------------------------------------------------------

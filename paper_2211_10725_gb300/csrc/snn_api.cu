@@ -278,19 +278,36 @@ snn_status_t scan_bwd(const snn_scan_desc* d, int neuron, const void* I, const f
   a.part_alpha = ((syn || rec) && grad_alpha) ? v.part[2] : nullptr;
   a.gmem0 = grad_mem0;
   a.gsyn0 = syn ? grad_syn0 : nullptr;
+  PartInfo info = {};  // PART_LANE unless a staged launch says otherwise
+  a.part_info = &info;
   const bool staged = staged_ok(d);
   cudaError_t e = syn ? launch_scan_bwd_synaptic(a, recompute, d->in_dtype, d->io_dtype, staged, stream)
                       : launch_scan_bwd_leaky(a, recompute, d->in_dtype, d->io_dtype, staged, stream);
   if (e != cudaSuccess) return cuda_status(e);
-  // one launch per parameter layout in use
+  // one launch per parameter layout in use (a layout's parameters share
+  // their partials' layout too: it depends on the mode alone)
   float* parts[3] = {a.part_beta, a.part_thr, a.part_alpha};
   for (int mode = SNN_P_SCALAR; mode <= SNN_P_PER_CHANNEL; ++mode) {
     ParamReduce jobs[3];
-    int n = 0;
+    int n = 0, kind = PART_LANE;
     for (int k = 0; k < 3; ++k)
-      if (outs[k] && modes[k] == mode) jobs[n++] = ParamReduce{parts[k], outs[k], v.scratch[k], v.tickets[k]};
+      if (outs[k] && modes[k] == mode) {
+        jobs[n++] = ParamReduce{parts[k], outs[k], v.scratch[k], v.tickets[k]};
+        kind = info.kind[k];
+      }
     if (n == 0) continue;
-    e = launch_param_reduce(jobs, n, d->B, d->N, d->C, d->HW, mode, red_scratch(d), stream);
+    int64_t B = d->B, N = d->N, HW = d->HW;
+    if (kind == PART_WARP) {
+      B = 1;
+      N = info.warps;
+    } else if (kind == PART_CHANNELS) {
+      B = 1;
+      N = info.warps * d->C;
+    } else if (kind == PART_RUN) {
+      N /= info.q;
+      HW /= info.q;
+    }
+    e = launch_param_reduce(jobs, n, B, N, d->C, HW, mode, red_scratch(d), stream);
     if (e != cudaSuccess) return SNN_ERR_CUDA;
   }
   return SNN_OK;

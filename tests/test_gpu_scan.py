@@ -480,3 +480,39 @@ def test_register_segment_recompute(case, neuron, cuda_device):
     if layer.ckpt is not None:  # T > K: checkpoints exist
         assert torch.equal(layer.ckpt, old.ckpt)
     H.assert_close("grad_I", H.lanes_2d(layer.grad_I), H.lanes_2d(old.grad_I), *H.TOL[w.io_dtype])
+
+
+# Staged scans over the shapes their strips and items can go wrong at: T
+# around the 4-step items and 8-step stages, more strips than resident CTAs,
+# a ragged last strip and warp; every layout the warps add partials in
+# (scalar, channel-last, runs of 32, 16 and 8 lanes, and channel counts and
+# run lengths that keep one partial per lane).  T, B, N, C, HW, mode, io,
+# neuron, reset.
+STRIP_CASES = [
+    (1, 2, 1000, 1, 1, "scalar", W.F32, "leaky", "subtract"),
+    (4, 3, 1008, 1, 1, "scalar", W.BF16, "leaky", "zero"),
+    (5, 70, 8192, 64, 1, "per_channel", W.BF16, "leaky", "zero"),
+    (8, 40, 16384, 16, 1024, "per_channel", W.F32, "leaky", "subtract"),
+    (25, 3, 12 * 48, 12, 48, "per_channel", W.BF16, "leaky", "zero"),
+    (13, 5, 6 * 40, 6, 40, "per_channel", W.F32, "synaptic", "subtract"),
+    (9, 6, 24 * 10, 24, 1, "per_channel", W.F16, "leaky", "subtract"),
+    (65, 2, 512, 128, 1, "per_channel", W.BF16, "rleaky", "subtract"),
+    (67, 9, 1032, 1, 1, "scalar", W.BF16, "synaptic", "zero"),
+    (66, 1, 8, 8, 1, "per_channel", W.F32, "rleaky", "subtract"),
+]
+
+
+@pytest.mark.parametrize("case", range(len(STRIP_CASES)))
+def test_strips_items_and_partials(case, cuda_device):
+    T, B, N, C, HW, mode, dt, neuron, reset = STRIP_CASES[case]
+    w = W.ScanWorkload(
+        name=f"strips_{case}", neuron=neuron, T=T, B=B, N=N, C=C, HW=HW, in_dtype=dt, io_dtype=dt,
+        i_mean=0.4, i_std=0.5, beta=("uniform", 0.6, 0.95), thr=("uniform", 0.7, 1.3),
+        alpha=("uniform", 0.5, 0.9), v=("uniform", -0.5, 0.3), beta_mode=mode, thr_mode=mode,
+        alpha_mode=mode, v_mode=mode, reset=reset, surrogate="fast_sigmoid", sg_param=5.0,
+        save="mem", want_mem=True, seed_index=900 + case)
+    inp = W.make_scan_inputs(w, with_mem0=case % 2 == 0, with_grad_mem=case % 3 == 0,
+                             with_grad_final=case % 2 == 1)
+    layer = H.run_gpu(w, inp)
+    assert layer.status() == 0
+    H.check_all(w, inp, layer, H.oracle_expect(w, inp))
