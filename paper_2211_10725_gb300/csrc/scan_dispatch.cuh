@@ -68,7 +68,7 @@ cudaError_t fwd_t(ScanArgs a, bool staged, cudaStream_t st) {
     if (launched || e != cudaSuccess) return e;
   }
   if (a.L == 0) return cudaSuccess;
-  return launch_pdl(scan_fwd_plain<SYN, TI, TO>, dim3((unsigned)ceil_div(a.L, 256)), dim3(256), 0,
+  return launch_pdl(scan_fwd_plain<SYN, TI, TO>, dim3((unsigned)ceil_div(a.L, 128)), dim3(128), 0,
                     st, a);
 }
 
