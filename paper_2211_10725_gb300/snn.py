@@ -136,16 +136,26 @@ def _check(status: int, where: str):
 
 
 def _ptr(t) -> Optional[int]:
-    if t is None:
-        return None
-    if isinstance(t, int):
+    if t is None or type(t) is int:
         return t
     return t.data_ptr()
 
 
+def _current_raw_stream() -> int:
+    """The current device's current stream.  torch.cuda.current_stream()
+    builds a Stream object for it, a third of a call's host time (2.9 us of
+    the 8.4 us of a Leaky forward; this takes 0.2 us)."""
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+
+
+if not (hasattr(torch._C, "_cuda_getCurrentRawStream") and hasattr(torch._C, "_cuda_getDevice")):
+    def _current_raw_stream() -> int:
+        return torch.cuda.current_stream().cuda_stream
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        return torch.cuda.current_stream().cuda_stream
+        return _current_raw_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -182,7 +192,7 @@ def snn_scan_ckpt_elems(desc: ScanDesc, synaptic: bool) -> int:
 
 
 def snn_workspace_init(ws: torch.Tensor, stream=None):
-    _check(load_library().snn_workspace_init(_ptr(ws), ws.numel() * ws.element_size(),
+    _check(load_library().snn_workspace_init(_ptr(ws), ws.nbytes,
                                              _stream(stream)), "snn_workspace_init")
 
 
@@ -193,7 +203,7 @@ def snn_workspace_status(ws: torch.Tensor, stream=None) -> int:
 def snn_leaky_fwd(desc, I, beta, thr, mem0, spk, mem, ckpt, mem_final, ws, stream=None):
     _check(load_library().snn_leaky_fwd(
         ctypes.byref(desc), _ptr(I), _ptr(beta), _ptr(thr), _ptr(mem0), _ptr(spk), _ptr(mem),
-        _ptr(ckpt), _ptr(mem_final), _ptr(ws), ws.numel() * ws.element_size(),
+        _ptr(ckpt), _ptr(mem_final), _ptr(ws), ws.nbytes,
         _stream(stream)), "snn_leaky_fwd")
 
 
@@ -203,7 +213,7 @@ def snn_leaky_bwd(desc, I, ckpt, mem, spk, beta, thr, mem0, grad_spk, grad_mem,
         ctypes.byref(desc), _ptr(I), _ptr(ckpt), _ptr(mem), _ptr(spk), _ptr(beta), _ptr(thr),
         _ptr(mem0), _ptr(grad_spk), _ptr(grad_mem), _ptr(grad_mem_final), _ptr(grad_I),
         _ptr(grad_beta), _ptr(grad_thr), _ptr(grad_mem0), _ptr(ws),
-        ws.numel() * ws.element_size(), _stream(stream)), "snn_leaky_bwd")
+        ws.nbytes, _stream(stream)), "snn_leaky_bwd")
 
 
 def snn_synaptic_fwd(desc, I, alpha, beta, thr, mem0, syn0, spk, mem, syn, ckpt, mem_final,
@@ -211,7 +221,7 @@ def snn_synaptic_fwd(desc, I, alpha, beta, thr, mem0, syn0, spk, mem, syn, ckpt,
     _check(load_library().snn_synaptic_fwd(
         ctypes.byref(desc), _ptr(I), _ptr(alpha), _ptr(beta), _ptr(thr), _ptr(mem0),
         _ptr(syn0), _ptr(spk), _ptr(mem), _ptr(syn), _ptr(ckpt), _ptr(mem_final),
-        _ptr(syn_final), _ptr(ws), ws.numel() * ws.element_size(), _stream(stream)),
+        _ptr(syn_final), _ptr(ws), ws.nbytes, _stream(stream)),
         "snn_synaptic_fwd")
 
 
@@ -223,13 +233,13 @@ def snn_synaptic_bwd(desc, I, ckpt, mem, spk, syn, alpha, beta, thr, mem0, syn0,
         _ptr(beta), _ptr(thr), _ptr(mem0), _ptr(syn0), _ptr(grad_spk), _ptr(grad_mem),
         _ptr(grad_mem_final), _ptr(grad_syn_final), _ptr(grad_I), _ptr(grad_alpha),
         _ptr(grad_beta), _ptr(grad_thr), _ptr(grad_mem0), _ptr(grad_syn0), _ptr(ws),
-        ws.numel() * ws.element_size(), _stream(stream)), "snn_synaptic_bwd")
+        ws.nbytes, _stream(stream)), "snn_synaptic_bwd")
 
 
 def snn_rleaky_fwd(desc, I, v, beta, thr, mem0, spk, mem, ckpt, mem_final, ws, stream=None):
     _check(load_library().snn_rleaky_fwd(
         ctypes.byref(desc), _ptr(I), _ptr(v), _ptr(beta), _ptr(thr), _ptr(mem0), _ptr(spk),
-        _ptr(mem), _ptr(ckpt), _ptr(mem_final), _ptr(ws), ws.numel() * ws.element_size(),
+        _ptr(mem), _ptr(ckpt), _ptr(mem_final), _ptr(ws), ws.nbytes,
         _stream(stream)), "snn_rleaky_fwd")
 
 
@@ -240,7 +250,7 @@ def snn_rleaky_bwd(desc, I, ckpt, mem, spk, v, beta, thr, mem0, grad_spk, grad_m
         ctypes.byref(desc), _ptr(I), _ptr(ckpt), _ptr(mem), _ptr(spk), _ptr(v), _ptr(beta),
         _ptr(thr), _ptr(mem0), _ptr(grad_spk), _ptr(grad_mem), _ptr(grad_mem_final),
         _ptr(grad_I), _ptr(grad_v), _ptr(grad_beta), _ptr(grad_thr), _ptr(grad_mem0), _ptr(ws),
-        ws.numel() * ws.element_size(), _stream(stream)), "snn_rleaky_bwd")
+        ws.nbytes, _stream(stream)), "snn_rleaky_bwd")
 
 
 def snn_leaky_bwd_noalloc(desc, I, ckpt, mem, spk, beta, thr, mem0, grad_spk, grad_mem,
@@ -264,7 +274,7 @@ def snn_dense_layer_fwd(X, W, I, ws, stream=None):
     M, K = X.shape[-2], X.shape[-1]
     N = W.shape[0]
     _check(load_library().snn_dense_layer_fwd(M, K, N, _ptr(X), _ptr(W), _ptr(I), _ptr(ws),
-                                              ws.numel() * ws.element_size(), _stream(stream)),
+                                              ws.nbytes, _stream(stream)),
            "snn_dense_layer_fwd")
 
 
@@ -273,7 +283,7 @@ def snn_dense_layer_bwd(X, W, dI, dX, dW, ws, stream=None):
     M, K = X.shape[-2], X.shape[-1]
     N = W.shape[0]
     _check(load_library().snn_dense_layer_bwd(M, K, N, _ptr(X), _ptr(W), _ptr(dI), _ptr(dX),
-                                              _ptr(dW), _ptr(ws), ws.numel() * ws.element_size(),
+                                              _ptr(dW), _ptr(ws), ws.nbytes,
                                               _stream(stream)), "snn_dense_layer_bwd")
 
 
@@ -335,7 +345,7 @@ def snn_rate_ce_loss(spk, labels, C, loss, grad_spk, ws=None, stream=None, batch
         ws = torch.zeros(snn_rate_ce_workspace_bytes(B), dtype=torch.uint8, device=spk.device)
     _check(load_library().snn_rate_ce_loss(T, B, C, pop, ld, batch_total or 0, dt, _ptr(spk),
                                            _ptr(labels), _ptr(loss), _ptr(grad_spk), _ptr(ws),
-                                           ws.numel() * ws.element_size(), _stream(stream)),
+                                           ws.nbytes, _stream(stream)),
            "snn_rate_ce_loss")
 
 
@@ -348,7 +358,7 @@ def snn_rate_ce_leaky_bwd(desc, spk, labels, C, beta, thr, mem, ckpt, loss, grad
                                                 _ptr(spk), _ptr(labels), _ptr(beta), _ptr(thr),
                                                 _ptr(mem), _ptr(ckpt), _ptr(loss), _ptr(grad_spk),
                                                 _ptr(grad_I), _ptr(ws),
-                                                ws.numel() * ws.element_size(), _stream(stream)),
+                                                ws.nbytes, _stream(stream)),
            "snn_rate_ce_leaky_bwd")
 
 
@@ -373,7 +383,7 @@ def snn_dense_leaky_fwd(desc, X, W, beta, thr, spk, mem, ckpt, ws, P=1, stream=N
     K = X.shape[-1]
     _check(load_library().snn_dense_leaky_fwd(ctypes.byref(desc), P, K, _ptr(X), _ptr(W),
                                               _ptr(beta), _ptr(thr), _ptr(spk), _ptr(mem),
-                                              _ptr(ckpt), _ptr(ws), ws.numel() * ws.element_size(),
+                                              _ptr(ckpt), _ptr(ws), ws.nbytes,
                                               _stream(stream)), "snn_dense_leaky_fwd")
 
 
@@ -384,7 +394,7 @@ def snn_dense_leaky_bwd(desc, dI_up, W, beta, thr, mem, spk, ckpt, grad_I, ws, s
     _check(load_library().snn_dense_leaky_bwd(ctypes.byref(desc), K, _ptr(dI_up), _ptr(W),
                                               _ptr(beta), _ptr(thr), _ptr(mem), _ptr(spk),
                                               _ptr(ckpt), _ptr(grad_I), _ptr(ws),
-                                              ws.numel() * ws.element_size(), _stream(stream)),
+                                              ws.nbytes, _stream(stream)),
            "snn_dense_leaky_bwd")
 
 
@@ -413,7 +423,7 @@ def snn_conv2d_small_dw_nhwc(X, dI, dW, KH, KW, ws, stream=None):
     Cout, ldw = dW.shape
     _check(load_library().snn_conv2d_small_dw_nhwc(M, H, W_, Cin, Cout, KH, KW, ldw, _ptr(X),
                                                    _ptr(dI), _ptr(dW), _ptr(ws),
-                                                   ws.numel() * ws.element_size(),
+                                                   ws.nbytes,
                                                    _stream(stream)), "snn_conv2d_small_dw_nhwc")
 
 
