@@ -63,6 +63,53 @@ struct GemmArgs {
   int64_t split_stride;  // elements between the partial outputs of two splits
 };
 
+// One warp's 32 rows of a finished accumulator to D as 128-byte column
+// chunks: TMEM -> registers -> swizzled staging -> TMA store (rows and
+// columns past M and N are clipped by the map).  acc: the warp's TMEM
+// address; returns the warp's chunk count (staging buffer parity).
+template <int BN, bool OUT_BF16>
+__device__ __forceinline__ int store_tile_chunks(const CUtensorMap& td, uint32_t acc, unsigned char* stage_out,
+                                                 int nchunk, int row0, int n0, int N, int sp, int lid) {
+  constexpr int OUT_CW = OUT_BF16 ? 64 : 32;  // columns of one 128-byte output chunk
+#pragma unroll 1
+  for (int c = 0; c < BN && n0 + c < N; c += OUT_CW) {
+    unsigned char* buf = stage_out + (nchunk & 1) * kOutChunkBytes;
+    if (lid == 0) bulk_wait_read_all_but_one();  // this buffer's last store has read it
+    __syncwarp();
+    unsigned char* rowp = buf + lid * 128;
+#pragma unroll
+    for (int cc = 0; cc < OUT_CW; cc += 16) {
+      uint32_t r[16];
+      tmem_ld16(acc + (uint32_t)(c + cc), r);
+      if (OUT_BF16) {
+        uint32_t w[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
+          w[j] = *reinterpret_cast<uint32_t*>(&h);
+        }
+        const int j0 = cc / 8;  // 16-byte chunk index of column cc within the row
+        *reinterpret_cast<uint4*>(rowp + (((j0) ^ (lid & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
+        *reinterpret_cast<uint4*>(rowp + (((j0 + 1) ^ (lid & 7)) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
+      } else {
+        const int j0 = cc / 4;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          *reinterpret_cast<uint4*>(rowp + (((j0 + j) ^ (lid & 7)) << 4)) =
+              make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
+      }
+    }
+    fence_async_smem();
+    __syncwarp();
+    if (lid == 0) {
+      tma_store_3d(&td, buf, n0 + c, row0, sp);
+      bulk_commit();
+    }
+    ++nchunk;
+  }
+  return nchunk;
+}
+
 // ---------------------------------------------------------------------------
 // Kernel: persistent, work items blockIdx.x, blockIdx.x + gridDim.x, ...;
 // item i is split i % S of tile i / S, tiles in row-major order (N tiles
@@ -216,44 +263,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
                                   : (void*)(static_cast<float*>(g.D) + sp * g.split_stride);
       const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN);
       if constexpr (TMA_OUT) {
-        // 128-byte column chunks: TMEM -> registers -> swizzled staging ->
-        // TMA store (rows and columns past M and N are clipped by the map)
-#pragma unroll 1
-        for (int c = 0; c < BN && n0 + c < g.N; c += OUT_CW) {
-          unsigned char* buf = stage_out + (nchunk & 1) * kOutChunkBytes;
-          if (lid == 0) bulk_wait_read_all_but_one();  // this buffer's last store has read it
-          __syncwarp();
-          unsigned char* rowp = buf + lid * 128;
-#pragma unroll
-          for (int cc = 0; cc < OUT_CW; cc += 16) {
-            uint32_t r[16];
-            tmem_ld16(acc + (uint32_t)(c + cc), r);
-            if (OUT_BF16) {
-              uint32_t w[8];
-#pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                __nv_bfloat162 h = __floats2bfloat162_rn(__uint_as_float(r[2 * j]), __uint_as_float(r[2 * j + 1]));
-                w[j] = *reinterpret_cast<uint32_t*>(&h);
-              }
-              const int j0 = cc / 8;  // 16-byte chunk index of column cc within the row
-              *reinterpret_cast<uint4*>(rowp + (((j0) ^ (lid & 7)) << 4)) = make_uint4(w[0], w[1], w[2], w[3]);
-              *reinterpret_cast<uint4*>(rowp + (((j0 + 1) ^ (lid & 7)) << 4)) = make_uint4(w[4], w[5], w[6], w[7]);
-            } else {
-              const int j0 = cc / 4;
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                *reinterpret_cast<uint4*>(rowp + (((j0 + j) ^ (lid & 7)) << 4)) =
-                    make_uint4(r[4 * j], r[4 * j + 1], r[4 * j + 2], r[4 * j + 3]);
-            }
-          }
-          fence_async_smem();
-          __syncwarp();
-          if (lid == 0) {
-            tma_store_3d(&td, buf, n0 + c, m0 + q * 32, sp);
-            bulk_commit();
-          }
-          ++nchunk;
-        }
+        nchunk = store_tile_chunks<BN, OUT_BF16>(td, acc, stage_out, nchunk, m0 + q * 32, n0, g.N, sp, lid);
       } else {
 #pragma unroll 1
       for (int c = 0; c < BN; c += 16) {
@@ -307,6 +317,191 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm)
 }
 
 // ---------------------------------------------------------------------------
+// CTA-pair kernel: two CTAs of a cluster work on one 256 x BN tile
+// (tcgen05.mma.cta_group::2).  Each loads its own 128 rows of A and half of
+// B's BN columns, so a CTA takes in 16 KB + 64*BN bytes a k-block for the
+// same 128 x BN outputs that cost a lone CTA 16 KB + 128*BN.  The lone
+// CTA's main loop was bound by that intake, not by the MMA: 128 x 256 tiles
+// need 96 bytes a clock per SM to keep the tensor core busy, and ran at
+// about 60% of its rate.  Everything else is the kernel above: persistent
+// work items, a ring that runs on across tiles, two accumulators, the
+// TMA-store epilogue.  The even CTA (the leader) issues every MMA; its
+// `full` barriers collect both CTAs' bytes and its `acc_empty` both CTAs'
+// epilogue warps, and its commits arrive on both CTAs' `empty` and
+// `acc_full`.
+// ---------------------------------------------------------------------------
+
+template <int BN>
+__host__ __device__ constexpr int pair_stages() { return 6; }
+template <int BN>
+__host__ __device__ constexpr size_t pair_smem_bytes() {
+  return 1024 + (size_t)pair_stages<BN>() * (BM * BK * 2 + BN / 2 * BK * 2) + kOutStaging + 256;
+}
+
+template <int BN, bool OUT_BF16, bool A_MN, bool B_MN>
+__global__ void __launch_bounds__(kThreads, 1)
+    gemm_pair_tcgen05(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
+                      const __grid_constant__ CUtensorMap td, const GemmArgs g) {
+  constexpr int HN = BN / 2;  // B columns this CTA loads
+  static_assert(BN % 32 == 0 && BN <= 256, "UMMA N for M = 256");
+  static_assert(!B_MN || HN % 64 == 0, "an MN-major B half is whole 64-wide boxes");
+  constexpr int OUT_CW = OUT_BF16 ? 64 : 32;
+  static_assert(BN % OUT_CW == 0, "the tile is whole output chunks");
+  constexpr int A_BYTES = BM * BK * 2;
+  constexpr int B_BYTES = HN * BK * 2;
+  constexpr uint32_t TCOLS = tmem_cols<BN>();
+  constexpr int kEpiWarps = 4;
+  constexpr int kStages = pair_stages<BN>();
+  static_assert(pair_smem_bytes<BN>() <= 227 * 1024, "the ring and staging fit one CTA");
+  extern __shared__ unsigned char smem_raw[];
+  unsigned char* smem =
+      reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  unsigned char* sA = smem;
+  unsigned char* sB = smem + kStages * A_BYTES;
+  unsigned char* sOut = sB + kStages * B_BYTES;
+  uint64_t* full = reinterpret_cast<uint64_t*>(sOut + kOutStaging);
+  uint64_t* empty = full + kStages;
+  uint64_t* acc_full = empty + kStages;
+  uint64_t* acc_empty = acc_full + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + 2);
+  const int warp = threadIdx.x >> 5, lid = threadIdx.x & 31;
+  const int rank = (int)cluster_rank();
+  const int pair = (int)blockIdx.x >> 1, pairs = (int)gridDim.x >> 1;
+  const int nk = (g.K + BK - 1) / BK;
+  const int tiles_n = (g.N + BN - 1) / BN;
+  const int S = g.ksplit;
+  const int items = tiles_n * ((g.M + 2 * BM - 1) / (2 * BM)) * S;
+
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&full[s], 1);
+      mbar_init(&empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&acc_full[b], 1);
+      mbar_init(&acc_empty[b], 2 * kEpiWarps);
+    }
+    fence_barrier_init();
+  }
+  if (warp == 1) tmem_alloc_pair(tmem_slot, TCOLS);
+  tc_fence_before();
+  __syncthreads();
+  cluster_barrier();  // both CTAs' barriers are initialised
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  grid_dep_wait();  // the previous kernel on the stream is complete
+
+  if (warp == 0) {
+    if (lid == 0) {
+      int64_t n_issued = 0;
+      bool ok = true;
+      for (int it = pair; it < items && ok; it += pairs) {
+        const int t = it / S, sp = it - t * S;
+        const int m0 = (t / tiles_n) * 2 * BM + rank * BM, n0 = (t % tiles_n) * BN + rank * HN;
+        const int kb1 = (int)((int64_t)nk * (sp + 1) / S);
+        for (int kb = (int)((int64_t)nk * sp / S); kb < kb1; ++kb, ++n_issued) {
+          const int s = (int)(n_issued % kStages);
+          if (n_issued >= kStages &&
+              !mbar_wait_poll(&empty[s], (uint32_t)(((n_issued / kStages) - 1) & 1), g.wait_ns)) {
+            record_status(g.status, kStatusTimeout);
+            ok = false;
+            break;
+          }
+          // the leader's barrier expects both CTAs' bytes (the peer's may
+          // land before the leader announces them)
+          if (rank == 0) mbar_arrive_expect_tx(&full[s], 2 * (A_BYTES + B_BYTES));
+          const uint32_t bar = cluster_addr(&full[s], 0);
+          if (A_MN) {
+#pragma unroll
+            for (int j = 0; j < BM / 64; ++j)
+              tma_load_2d_pair(sA + s * A_BYTES + j * kMnBoxBytes, &ta, m0 + 64 * j, kb * BK, bar);
+          } else {
+            tma_load_2d_pair(sA + s * A_BYTES, &ta, kb * BK, m0, bar);
+          }
+          if (B_MN) {
+#pragma unroll
+            for (int j = 0; j < HN / 64; ++j)
+              tma_load_2d_pair(sB + s * B_BYTES + j * kMnBoxBytes, &tb, n0 + 64 * j, kb * BK, bar);
+          } else {
+            tma_load_2d_pair(sB + s * B_BYTES, &tb, kb * BK, n0, bar);
+          }
+        }
+      }
+      // every copy has landed before the CTAs may exit: the leader's barriers
+      // count both CTAs' copies
+      if (rank == 0)
+        for (int64_t j = n_issued > kStages ? n_issued - kStages : 0; j < n_issued; ++j)
+          mbar_wait_bounded(&full[j % kStages], (uint32_t)((j / kStages) & 1), kDrainWaitNs);
+    }
+  } else if (warp == 1) {
+    if (rank == 0 && lid == 0) {
+      constexpr uint32_t idesc = idesc_bf16(2 * BM, BN, A_MN, B_MN);
+      constexpr uint64_t stepA = A_MN ? 2048 >> 4 : 32 >> 4;
+      constexpr uint64_t stepB = B_MN ? 2048 >> 4 : 32 >> 4;
+      int64_t n_used = 0;
+      bool ok = true;
+      int i = 0;
+      for (int it = pair; it < items && ok; it += pairs, ++i) {
+        const int sp = it % S;
+        const int kb0 = (int)((int64_t)nk * sp / S), kb1 = (int)((int64_t)nk * (sp + 1) / S);
+        const int b = i & 1;
+        if (i >= 2 && !mbar_wait_poll(&acc_empty[b], (uint32_t)(((i >> 1) - 1) & 1), g.wait_ns)) {
+          record_status(g.status, kStatusTimeout);
+          break;
+        }
+        tc_fence_after();
+        const uint32_t acc = tmem + (uint32_t)(b * BN);
+        for (int kb = kb0; kb < kb1; ++kb, ++n_used) {
+          const int s = (int)(n_used % kStages);
+          if (!mbar_wait_poll(&full[s], (uint32_t)((n_used / kStages) & 1), g.wait_ns)) {
+            record_status(g.status, kStatusTimeout);
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint64_t da = A_MN ? sdesc_sw128_mn(sA + s * A_BYTES) : sdesc_sw128(sA + s * A_BYTES);
+          const uint64_t db = B_MN ? sdesc_sw128_mn(sB + s * B_BYTES) : sdesc_sw128(sB + s * B_BYTES);
+#pragma unroll
+          for (int kk = 0; kk < BK / 16; ++kk)
+            tc_mma_pair(acc, da + stepA * kk, db + stepB * kk, idesc, (kb != kb0 || kk != 0) ? 1u : 0u);
+          tc_commit_pair(&empty[s]);  // both CTAs' stages are free once these MMAs are done
+        }
+        if (ok) tc_commit_pair(&acc_full[b]);
+      }
+    }
+  } else {
+    const int q = warp & 3;
+    unsigned char* stage_out = sOut + q * 2 * kOutChunkBytes;
+    int nchunk = 0;
+    int i = 0;
+    for (int it = pair; it < items; it += pairs, ++i) {
+      const int t = it / S, sp = it - t * S;
+      const int b = i & 1;
+      if (!warp_wait_uniform(&acc_full[b], (uint32_t)((i >> 1) & 1), g.wait_ns)) {
+        if (lid == 0) record_status(g.status, kStatusTimeout);
+        break;
+      }
+      tc_fence_after();
+      const int m0 = (t / tiles_n) * 2 * BM + rank * BM, n0 = (t % tiles_n) * BN;
+      const uint32_t acc = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(b * BN);
+      if (m0 + q * 32 < g.M)  // whole warps of rows past M have nothing to store
+        nchunk = store_tile_chunks<BN, OUT_BF16>(td, acc, stage_out, nchunk, m0 + q * 32, n0, g.N, sp, lid);
+      tc_fence_before();
+      __syncwarp();
+      if (lid == 0) mbar_arrive_cluster(&acc_empty[b], 0);
+    }
+    if (lid == 0) bulk_wait_all();  // the staged chunks are written out
+  }
+  tc_fence_before();
+  __syncthreads();
+  cluster_barrier();  // neither CTA leaves while the other may still signal it
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc_pair(tmem, TCOLS);
+  }
+}
+
+// ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
 
@@ -343,6 +538,59 @@ cudaError_t launch_out(const CUtensorMap& ta, const CUtensorMap& tb, const GemmA
   return launch_bn<BN, OUT_BF16, A_MN, B_MN, false>(ta, tb, td, g, st);
 }
 
+// ---- CTA pairs ------------------------------------------------------------
+
+// Clocks of one k-block of a work item: the tensor core takes 2*bn (4096
+// multiply-adds a clock for 128 rows), and the SM takes in about 60 bytes a
+// clock (measured: 128 x 256 tiles at 6400 x 3072 x 1000 ran two rounds of
+// 48 k-blocks in 39 us).
+inline int64_t kblock_clocks(int bn, bool pair) {
+  const int64_t feed = (BM * BK * 2 + (int64_t)bn * BK * (pair ? 1 : 2)) / 60;
+  return feed > 2 * bn ? feed : 2 * bn;
+}
+
+// Width of the CTA-pair tile for a product that would take `bn`-wide tiles
+// on single CTAs, or 0 for those: the width that minimises rounds of work
+// items times a k-block's clocks, where that saves a tenth or more, the
+// product has more rows than one CTA's 128 and each item has at least 16
+// k-blocks (below that the fill and the epilogue decide, and the pair's are
+// longer by the cluster's start: the 1000 x 1000 weight gradient over 3200
+// rows, 12 k-blocks an item, took 15.0 us against 14.4).  6400 x 3072 x
+// 1000, the three products of a pass back to back: 119 -> 100 us (the input
+// gradient alone 41 -> 31.5 us; 62 us at 1.9 PFLOP/s).
+template <bool OUT_BF16, bool B_MN>
+int pair_width(int M, int N, int K, int S, int bn, int sms) {
+  if (sms < 2 || M <= BM || (K + BK - 1) / BK / S < 16) return 0;
+  auto rounds = [](int64_t items, int64_t units) { return (items + units - 1) / units; };
+  const int64_t one = rounds((int64_t)((N + bn - 1) / bn) * ((M + BM - 1) / BM) * S, sms) *
+                      kblock_clocks(bn, false);
+  int64_t best = one - one / 10;
+  int width = 0;
+  const int cand[3] = {256, B_MN ? 0 : 192, 128};
+  for (int w : cand) {
+    if (w == 0) continue;
+    const int64_t items = (int64_t)((N + w - 1) / w) * ((M + 2 * BM - 1) / (2 * BM)) * S;
+    const int64_t c = rounds(items, sms / 2) * kblock_clocks(w, true);
+    if (c < best) {
+      best = c;
+      width = w;
+    }
+  }
+  return width;
+}
+
+template <int BN, bool OUT_BF16, bool A_MN, bool B_MN>
+cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const CUtensorMap& td, const GemmArgs& g,
+                        int sms, cudaStream_t st) {
+  const void* k = (const void*)gemm_pair_tcgen05<BN, OUT_BF16, A_MN, B_MN>;
+  const cudaError_t e = ensure_smem(k, pair_smem_bytes<BN>());
+  if (e != cudaSuccess) return e;
+  const int64_t items = (int64_t)((g.N + BN - 1) / BN) * ((g.M + 2 * BM - 1) / (2 * BM)) * g.ksplit;
+  const int64_t pairs = items < sms / 2 ? items : sms / 2;
+  return launch_pdl_cluster(2u, gemm_pair_tcgen05<BN, OUT_BF16, A_MN, B_MN>, dim3((unsigned)(2 * pairs)),
+                            dim3(kThreads), pair_smem_bytes<BN>(), st, ta, tb, td, g);
+}
+
 // D[M, N] = A[M, K] * B[N, K]^T.  A is stored [M, K] row-major (K-major) or,
 // with A_MN, [K, M] row-major; B likewise [N, K] or, with B_MN, [K, N].
 // N tile: the widest the output needs (64, 128 or 192 for an MN-major B),
@@ -370,6 +618,20 @@ cudaError_t gemm_tn(const void* A, const void* B, void* D, int M, int N, int K, 
   }
   CUtensorMap ta, tb;
   const bool okA = A_MN ? make_map(&ta, A, K, M, 64) : make_map(&ta, A, M, K, BM);
+  DeviceInfo info;
+  if (device_info(&info) == cudaSuccess && ((int64_t)N * (OUT_BF16 ? 2 : 4)) % 16 == 0 &&
+      (reinterpret_cast<uintptr_t>(D) & 15u) == 0) {
+    const int w = pair_width<OUT_BF16, B_MN>(M, N, K, ksplit, bn, info.sms);
+    CUtensorMap td;
+    if (w > 0 && okA && (B_MN ? make_map(&tb, B, K, N, 64) : make_map(&tb, B, N, K, w / 2)) &&
+        make_out_map(&td, D, ksplit, M, N, OUT_BF16)) {
+      const GemmArgs g{M, N, K, D, (int64_t)N, status, kDefaultWaitNs, ksplit, (int64_t)M * N};
+      if (w == 256) return launch_pair<256, OUT_BF16, A_MN, B_MN>(ta, tb, td, g, info.sms, st);
+      if constexpr (!B_MN)
+        if (w == 192) return launch_pair<192, OUT_BF16, A_MN, B_MN>(ta, tb, td, g, info.sms, st);
+      return launch_pair<128, OUT_BF16, A_MN, B_MN>(ta, tb, td, g, info.sms, st);
+    }
+  }
   const bool okB = B_MN ? make_map(&tb, B, K, N, 64) : make_map(&tb, B, N, K, bn);
   if (!okA || !okB) return cudaErrorInvalidValue;
   GemmArgs g{M, N, K, D, (int64_t)N, status, kDefaultWaitNs, ksplit, (int64_t)M * N};
