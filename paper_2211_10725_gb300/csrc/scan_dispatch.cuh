@@ -56,6 +56,12 @@ cudaError_t fwd_staged(ScanArgs a, cudaStream_t st, bool* launched) {
   return fwd_staged_vl<SYN, TI, TO, RESET, REC, kLanes<SYN>, false>(a, st, launched);
 }
 
+template <bool SYN, typename TI, typename TO, int RESET, int REC>
+cudaError_t fwd_plain(ScanArgs a, cudaStream_t st) {
+  return launch_pdl(scan_fwd_plain<SYN, TI, TO, RESET, REC>, dim3((unsigned)ceil_div(a.L, 128)), dim3(128),
+                    0, st, a);
+}
+
 template <bool SYN, typename TI, typename TO>
 cudaError_t fwd_t(ScanArgs a, bool staged, cudaStream_t st) {
   if (staged && a.L > 0) {
@@ -68,8 +74,11 @@ cudaError_t fwd_t(ScanArgs a, bool staged, cudaStream_t st) {
     if (launched || e != cudaSuccess) return e;
   }
   if (a.L == 0) return cudaSuccess;
-  return launch_pdl(scan_fwd_plain<SYN, TI, TO>, dim3((unsigned)ceil_div(a.L, 128)), dim3(128), 0,
-                    st, a);
+  if constexpr (!SYN)
+    if (a.rec) return fwd_plain<SYN, TI, TO, RESET_SUBTRACT, 1>(a, st);
+  if (a.reset == RESET_SUBTRACT) return fwd_plain<SYN, TI, TO, RESET_SUBTRACT, 0>(a, st);
+  if (a.reset == RESET_ZERO) return fwd_plain<SYN, TI, TO, RESET_ZERO, 0>(a, st);
+  return fwd_plain<SYN, TI, TO, RESET_NONE, 0>(a, st);
 }
 
 template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int KC, bool REC,
@@ -115,6 +124,16 @@ cudaError_t bwd_staged(ScanArgs a, cudaStream_t st, bool* launched) {
   return bwd_staged_vl<SYN, RECOMP, TI, TO, RESET, SG, KC, REC, kLanes<SYN>>(a, st, launched);
 }
 
+template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int REC>
+cudaError_t bwd_plain(ScanArgs a, cudaStream_t st) {
+  const int threads = 128;
+  const size_t smem = RECOMP ? (size_t)a.K * threads * 4 * (SYN ? 2 : 1) : 0;
+  const cudaError_t e = ensure_smem((const void*)scan_bwd_plain<SYN, RECOMP, TI, TO, RESET, SG, REC>, smem);
+  if (e != cudaSuccess) return e;
+  return launch_pdl(scan_bwd_plain<SYN, RECOMP, TI, TO, RESET, SG, REC>,
+                    dim3((unsigned)ceil_div(a.L, threads)), dim3(threads), smem, st, a);
+}
+
 template <bool SYN, bool RECOMP, typename TI, typename TO>
 cudaError_t bwd_t(ScanArgs a, bool staged, cudaStream_t st) {
   if (staged && a.L > 0) {
@@ -158,13 +177,23 @@ cudaError_t bwd_t(ScanArgs a, bool staged, cudaStream_t st) {
     if (launched || e != cudaSuccess) return e;
   }
   if (a.L == 0) return cudaSuccess;
-  const int threads = 128;
-  const size_t smem = RECOMP ? (size_t)a.K * threads * 4 * (SYN ? 2 : 1) : 0;
-  const void* k = (const void*)scan_bwd_plain<SYN, RECOMP, TI, TO>;
-  cudaError_t e = ensure_smem(k, smem);
-  if (e != cudaSuccess) return e;
-  return launch_pdl(scan_bwd_plain<SYN, RECOMP, TI, TO>, dim3((unsigned)ceil_div(a.L, threads)),
-                    dim3(threads), smem, st, a);
+  // the modes of a ragged layer: a warp has a scheduler nearly to itself, so
+  // every instruction of a step shows; run-time modes only for the mixed
+  // input and storage types and for no reset
+  if constexpr (std::is_same<TI, TO>::value) {
+    const bool atan = a.sg == SG_ATAN;
+    if constexpr (!SYN)
+      if (a.rec)
+        return atan ? bwd_plain<SYN, RECOMP, TI, TO, RESET_SUBTRACT, SG_ATAN, 1>(a, st)
+                    : bwd_plain<SYN, RECOMP, TI, TO, RESET_SUBTRACT, SG_FAST_SIGMOID, 1>(a, st);
+    if (a.reset == RESET_SUBTRACT)
+      return atan ? bwd_plain<SYN, RECOMP, TI, TO, RESET_SUBTRACT, SG_ATAN, 0>(a, st)
+                  : bwd_plain<SYN, RECOMP, TI, TO, RESET_SUBTRACT, SG_FAST_SIGMOID, 0>(a, st);
+    if (a.reset == RESET_ZERO)
+      return atan ? bwd_plain<SYN, RECOMP, TI, TO, RESET_ZERO, SG_ATAN, 0>(a, st)
+                  : bwd_plain<SYN, RECOMP, TI, TO, RESET_ZERO, SG_FAST_SIGMOID, 0>(a, st);
+  }
+  return bwd_plain<SYN, RECOMP, TI, TO, -1, -1, -1>(a, st);
 }
 
 // dtype codes (snn_dtype_t): 0 f32, 1 bf16, 2 f16.  Instantiated pairs

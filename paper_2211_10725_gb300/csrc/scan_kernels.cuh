@@ -185,16 +185,17 @@ struct BwdLane {
 // parameter terms of step t+1 that need the step-t state
 // (d u_{t+1}/d beta = u_t or (1-z_t) u_t, the subtract reset's -z_t, and
 // d i_{t+1}/d alpha = i_t), then the adjoint of step t.  Returns dL/dI_t.
-template <bool SYN, int RESET, int SG>
+template <bool SYN, int RESET, int SG, int REC = -1>  // REC -1: a.rec decides
 __device__ __forceinline__ float bwd_step(const ScanArgs& a, float beta, float thr, float alpha,
                                           bool has_next, float u, bool z, float i, float gs,
                                           float extra_u, float extra_i, BwdLane& s) {
   const int reset = RESET >= 0 ? RESET : a.reset;
+  const bool rec = !SYN && (REC >= 0 ? REC != 0 : a.rec != 0);
   if (has_next) {
     s.dbeta = fmaf(s.du, (reset == RESET_ZERO && z) ? 0.0f : u, s.dbeta);
     if (reset == RESET_SUBTRACT && z) s.dthr -= s.du;
     if (SYN) s.dalpha = fmaf(s.di, i, s.dalpha);
-    if (!SYN && a.rec && z) s.dalpha += s.du;  // dv: d u_{t+1} / d v = z_t
+    if (rec && z) s.dalpha += s.du;  // dv: d u_{t+1} / d v = z_t
   }
   const float sgv = surrogate<SG>(a, u - thr);
   float dz = gs;
@@ -202,7 +203,7 @@ __device__ __forceinline__ float bwd_step(const ScanArgs& a, float beta, float t
     if (reset == RESET_SUBTRACT) dz = fmaf(-thr, s.du, dz);
     else if (reset == RESET_ZERO) dz = fmaf(-beta * u, s.du, dz);
   }
-  if (!SYN && a.rec) dz = fmaf(alpha, s.du, dz);  // the recurrent connection, never detached
+  if (rec) dz = fmaf(alpha, s.du, dz);  // the recurrent connection, never detached
   const float decay = (reset == RESET_ZERO && z) ? 0.0f : beta;
   const float du = fmaf(decay, s.du, fmaf(sgv, dz, extra_u));
   s.dthr = fmaf(-sgv, dz, s.dthr);
@@ -1227,7 +1228,8 @@ __device__ __forceinline__ void plain_steps(int64_t n, Load load, Step step) {
   }
 }
 
-template <bool SYN, typename TI, typename TO>
+// RESET, REC (and SG below): compile-time, or -1 for the run-time value.
+template <bool SYN, typename TI, typename TO, int RESET, int REC>
 __global__ void __launch_bounds__(128) scan_fwd_plain(const ScanArgs a) {
   grid_dep_wait();
   const int64_t l = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1238,7 +1240,7 @@ __global__ void __launch_bounds__(128) scan_fwd_plain(const ScanArgs a) {
   float u = a.mem0 ? a.mem0[l] : 0.0f;
   bool z = a.mem0 ? (u > thr) : false;
   float i = (SYN && a.syn0) ? a.syn0[l] : 0.0f;
-  const TI* I = static_cast<const TI*>(a.I) + l;
+  const TI* I = static_cast<const TI*>(a.I) + l;  // walks forward: loads come in order
   TO* spk = static_cast<TO*>(a.spk) + l;
   TO* mem = a.mem ? static_cast<TO*>(a.mem) + l : nullptr;
   TO* syn = (SYN && a.syn) ? static_cast<TO*>(a.syn) + l : nullptr;
@@ -1246,13 +1248,24 @@ __global__ void __launch_bounds__(128) scan_fwd_plain(const ScanArgs a) {
   int kk = a.nseg > 0 ? seg_phase0(a) : 0;
   float* cp = a.ckpt ? a.ckpt + l : nullptr;
   plain_steps<TI>(
-      a.T, [&](int64_t t) { return I[t * a.L]; },
+      a.T,
+      [&](int64_t) {
+        const TI x = *I;
+        I += a.L;
+        return x;
+      },
       [&](int64_t t, const TI& x) {
-        const int64_t off = t * a.L;
-        fwd_step<SYN, -1, -1>(a.reset, beta, thr, alpha, Elem<TI>::load1(&x), u, z, i, a.rec != 0);
-        Elem<TO>::store1(spk + off, z ? 1.0f : 0.0f);
-        if (mem) Elem<TO>::store1(mem + off, u);
-        if (SYN && syn) Elem<TO>::store1(syn + off, i);
+        fwd_step<SYN, RESET, REC>(a.reset, beta, thr, alpha, Elem<TI>::load1(&x), u, z, i, a.rec != 0);
+        Elem<TO>::store1(spk, z ? 1.0f : 0.0f);
+        spk += a.L;
+        if (mem) {
+          Elem<TO>::store1(mem, u);
+          mem += a.L;
+        }
+        if (SYN && syn) {
+          Elem<TO>::store1(syn, i);
+          syn += a.L;
+        }
         if (++kk == a.K) {
           kk = 0;
           if (cp && t + 1 < a.T) {
@@ -1266,7 +1279,7 @@ __global__ void __launch_bounds__(128) scan_fwd_plain(const ScanArgs a) {
   if (SYN && a.syn_final) a.syn_final[l] = i;
 }
 
-template <bool SYN, bool RECOMP, typename TI, typename TO>
+template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int REC>
 __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
   extern __shared__ __align__(16) float segbuf[];  // [K][blockDim] u, then i
   grid_dep_wait();
@@ -1287,22 +1300,26 @@ __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
   TO* gI = static_cast<TO*>(a.gI) + l;
   BwdLane st{0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
   if (!RECOMP) {
+    // offset of the next step to load (they come in order, t = T-1 first) and
+    // the next to store
     const TO* mem = static_cast<const TO*>(a.mem_in) + l;
     const TO* spk = static_cast<const TO*>(a.spk_in) + l;
     const TO* syn = static_cast<const TO*>(a.syn_in) + l;
+    int64_t off = (a.T - 1) * a.L;
+    gI += off;
     struct Item {
       TO g, u, z, i, m;
     };
     plain_steps<Item>(
         a.T,
-        [&](int64_t k) {
-          const int64_t off = (a.T - 1 - k) * a.L;
+        [&](int64_t) {
           Item it;
           it.g = gs[off];
           it.u = mem[off];
           if (half_store) it.z = spk[off];
           if (want_syn) it.i = syn[off];
           if (gm) it.m = gm[off];
+          off -= a.L;
           return it;
         },
         [&](int64_t k, const Item& it) {
@@ -1311,9 +1328,10 @@ __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
           const bool z = half_store ? (Elem<TO>::load1(&it.z) != 0.0f) : (u > thr);
           const float i = want_syn ? Elem<TO>::load1(&it.i) : 0.0f;
           const float eu = (gm ? Elem<TO>::load1(&it.m) : 0.0f) + (last ? ex_u : 0.0f);
-          Elem<TO>::store1(gI + (a.T - 1 - k) * a.L,
-                           bwd_step<SYN, -1, -1>(a, beta, thr, alpha, !last, u, z, i,
-                                                 Elem<TO>::load1(&it.g), eu, last ? ex_i : 0.0f, st));
+          Elem<TO>::store1(gI, bwd_step<SYN, RESET, SG, REC>(a, beta, thr, alpha, !last, u, z, i,
+                                                             Elem<TO>::load1(&it.g), eu,
+                                                             last ? ex_i : 0.0f, st));
+          gI -= a.L;
         });
   } else {
     const TI* I = static_cast<const TI*>(a.I) + l;
@@ -1340,7 +1358,7 @@ __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
       plain_steps<TI>(
           t1 - t0, [&](int64_t j) { return I[(t0 + j) * a.L]; },
           [&](int64_t j, const TI& x) {
-            fwd_step<SYN, -1, -1>(a.reset, beta, thr, alpha, Elem<TI>::load1(&x), u, z, i, a.rec != 0);
+            fwd_step<SYN, RESET, REC>(a.reset, beta, thr, alpha, Elem<TI>::load1(&x), u, z, i, a.rec != 0);
             su[j * blockDim.x] = u;
             if (SYN) si[j * blockDim.x] = i;
           });
@@ -1360,7 +1378,7 @@ __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
             const bool last = (t == a.T - 1);
             const float eu = (gm ? Elem<TO>::load1(&it.m) : 0.0f) + (last ? ex_u : 0.0f);
             Elem<TO>::store1(gI + t * a.L,
-                             bwd_step<SYN, -1, -1>(a, beta, thr, alpha, !last, uu, uu > thr, iv,
+                             bwd_step<SYN, RESET, SG, REC>(a, beta, thr, alpha, !last, uu, uu > thr, iv,
                                                    Elem<TO>::load1(&it.g), eu, last ? ex_i : 0.0f, st));
           });
     }
