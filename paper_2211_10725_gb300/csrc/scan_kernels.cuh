@@ -22,6 +22,8 @@
 // they give bit-identical forward results.
 #pragma once
 
+#include <type_traits>
+
 #include "launch.cuh"
 #include "snn_device.cuh"
 
@@ -752,7 +754,8 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanA
 // [syn], [grad_mem]} (with one step per item the barriers' rate, not the
 // bytes in flight, bounded the half-precision scans: with 4, and 4 lanes a
 // thread, the recurrent neuron's two passes at T = 100 over 64 x 4096 lanes
-// in bf16 went from 90 to 72 us; 46 us at 6.8 TB/s).  Recompute
+// in bf16 went from 90 to 72 us, and with the whole items below free of
+// per-step tests to 68; 46 us at 6.8 TB/s).  Recompute
 // mode: checkpoint segments from last to first; per segment, items for
 // t = t0..t1-1 holding {I, [ckpt u, ckpt i at t0]} replay the forward into a
 // per-thread shared-memory buffer, then items t = t1-1..t0 holding
@@ -932,10 +935,65 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_bwd_staged(const ScanA
   };
 
   if (!RECOMP) {
-    // the final state's gradients enter at t = T-1 and are zero below it
+    // One reverse step on the tiles at byte `off` of the ring (the step's
+    // grad_spk; the other tiles follow io_stride apart), EXTRA: with eu / ei.
     float2 eu[NP], ei[NP];
 #pragma unroll
     for (int k = 0; k < NP; ++k) eu[k] = ei[k] = f2(0.0f);
+    const int bits_off = t_spk * io_stride + bits_skew + (V == 4 ? c / 2 : c) - c * V * (int)sizeof(TO);
+    const int bits_shift = V == 4 ? (c & 1) * 4 : 0;
+    auto step = [&](int off, TO* out_row, auto with_bits, auto extra) {
+      constexpr bool BITS = decltype(with_bits)::value, EXTRA = decltype(extra)::value;
+      float2 g[NP], uu[NP], ii[NP], out[NP];
+      bool zz[V];
+      const unsigned char* p = ring + off;
+      load_pairs<TO, NP>(reinterpret_cast<const TO*>(p), g);
+      load_pairs<TO, NP>(reinterpret_cast<const TO*>(p + io_stride), uu);
+      if constexpr (BITS) {
+        const unsigned zb = (unsigned)p[bits_off] >> bits_shift;
+#pragma unroll
+        for (int k = 0; k < V; ++k) zz[k] = (zb >> k) & 1u;
+      } else if constexpr (sizeof(TO) != 4) {
+        float2 sp[NP];
+        load_pairs<TO, NP>(reinterpret_cast<const TO*>(p + t_spk * io_stride), sp);
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+          zz[2 * k] = sp[k].x != 0.0f;
+          zz[2 * k + 1] = sp[k].y != 0.0f;
+        }
+      } else {
+#pragma unroll
+        for (int k = 0; k < NP; ++k) {
+          zz[2 * k] = uu[k].x > -negthr[k].x;
+          zz[2 * k + 1] = uu[k].y > -negthr[k].y;
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < NP; ++k) ii[k] = f2(0.0f);
+      if (want_syn) load_pairs<TO, NP>(reinterpret_cast<const TO*>(p + t_syn * io_stride), ii);
+      if constexpr (EXTRA) {
+        if (a.gm) {
+          float2 gmv[NP];
+          load_pairs<TO, NP>(reinterpret_cast<const TO*>(p + t_gm_store * io_stride), gmv);
+#pragma unroll
+          for (int k = 0; k < NP; ++k) eu[k] = add2(eu[k], gmv[k]);
+        }
+      }
+      bwd_pairs<SYN, RESET, SG, EXTRA, NP, REC>(a, beta, negthr, alpha, uu, zz, ii, g, eu, ei, st, out);
+      if constexpr (EXTRA) {
+#pragma unroll
+        for (int k = 0; k < NP; ++k) eu[k] = ei[k] = f2(0.0f);
+      }
+      store_pairs<TO, NP>(out_row, out);
+    };
+    // A whole item without per-step gradients is kBwdRows steps with no test
+    // in them (a step's tests and addresses were 10 of the 24 instructions a
+    // neuron-step took with 4 lanes a thread, and these scans in half
+    // precision are bound by issue slots); the first item when the final
+    // state's gradients enter at t = T-1, the last when T is no multiple, and
+    // every item with dL/dmem go step by step.
+    const int step_bytes = step_tiles * io_stride;
+    const bool finals = a.gmf || (SYN && a.gsf);
     if (active && a.gmf) load_pairs_global<NP>(a.gmf + l, eu);
     if (SYN && active && a.gsf) load_pairs_global<NP>(a.gsf + l, ei);
     for (int64_t t1 = a.T - 1; t1 >= 0; t1 -= kBwdRows) {
@@ -944,57 +1002,30 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_bwd_staged(const ScanA
         ok = false;
         break;
       }
-      const int nr = (int)min((int64_t)kBwdRows, t1 + 1);
       if (active) {
-        const TO* base = ring_o + pos.s * stage_io_elems;
+        const int base = pos.s * a.stage_bytes + c * V * (int)sizeof(TO);
+        const int64_t L = a.L;
+        if (t1 >= kBwdRows - 1 && !a.gm && !(finals && t1 == a.T - 1)) {
+          if (sizeof(TO) != 4 && use_bits) {
 #pragma unroll
-        for (int r = 0; r < kBwdRows; ++r) {
-          if (r < nr) {
-            float2 g[NP], uu[NP], ii[NP], gmv[NP], out[NP];
-            bool zz[V];
-            load_pairs<TO, NP>(base, g);
-            load_pairs<TO, NP>(base + tile_io_elems, uu);
-            if (use_bits) {
-              const unsigned char* bb = reinterpret_cast<const unsigned char*>(base - c * V) +
-                                        t_spk * io_stride + bits_skew + (V == 4 ? c / 2 : c);
-              const unsigned zb = V == 4 ? (unsigned)(*bb >> ((c & 1) * 4)) : (unsigned)*bb;
+            for (int r = 0; r < kBwdRows; ++r)
+              step(base + r * step_bytes, gI - r * L, std::true_type(), std::false_type());
+          } else {
 #pragma unroll
-              for (int k = 0; k < V; ++k) zz[k] = (zb >> k) & 1u;
-            } else if (half_store) {
-              float2 sp[NP];
-              load_pairs<TO, NP>(base + t_spk * tile_io_elems, sp);
-#pragma unroll
-              for (int k = 0; k < NP; ++k) {
-                zz[2 * k] = sp[k].x != 0.0f;
-                zz[2 * k + 1] = sp[k].y != 0.0f;
-              }
-            } else {
-#pragma unroll
-              for (int k = 0; k < NP; ++k) {
-                zz[2 * k] = uu[k].x > -negthr[k].x;
-                zz[2 * k + 1] = uu[k].y > -negthr[k].y;
-              }
-            }
-            if (want_syn) {
-              load_pairs<TO, NP>(base + t_syn * tile_io_elems, ii);
-            } else {
-#pragma unroll
-              for (int k = 0; k < NP; ++k) ii[k] = f2(0.0f);
-            }
-            if (a.gm) {
-              load_pairs<TO, NP>(base + t_gm_store * tile_io_elems, gmv);
-#pragma unroll
-              for (int k = 0; k < NP; ++k) eu[k] = add2(eu[k], gmv[k]);
-            }
-            bwd_pairs<SYN, RESET, SG, true, NP, REC>(a, beta, negthr, alpha, uu, zz, ii, g, eu, ei,
-                                                     st, out);
-#pragma unroll
-            for (int k = 0; k < NP; ++k) eu[k] = ei[k] = f2(0.0f);
-            store_pairs<TO, NP>(gI, out);
-            gI -= a.L;
-            base += step_tiles * tile_io_elems;
+            for (int r = 0; r < kBwdRows; ++r)
+              step(base + r * step_bytes, gI - r * L, std::false_type(), std::false_type());
+          }
+        } else {
+          const int nr = (int)min((int64_t)kBwdRows, t1 + 1);
+#pragma unroll 1
+          for (int r = 0; r < nr; ++r) {
+            if (sizeof(TO) != 4 && use_bits)
+              step(base + r * step_bytes, gI - r * L, std::true_type(), std::true_type());
+            else
+              step(base + r * step_bytes, gI - r * L, std::false_type(), std::true_type());
           }
         }
+        gI -= kBwdRows * L;
       }
       release_stage(empty, pos.s, lid);
       pos.next(S);
