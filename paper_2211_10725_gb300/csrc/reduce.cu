@@ -20,6 +20,8 @@
 // and writes the result, then resets the group's ticket to zero for the
 // next call.  Per neuron, a neuron's B partials fit one block, which sums
 // them in a single pass.
+#include <climits>
+
 #include "scan_host.cuh"
 
 namespace snn {
@@ -50,17 +52,24 @@ __device__ __forceinline__ float pair_value(float2 a) {
   return isfinite(a.x) ? __fadd_rn(a.x, a.y) : a.x;
 }
 
-// The block's values added in a fixed tree.
+// The lanes' values added in a fixed tree, in every lane.
+__device__ __forceinline__ float2 warp_sum_pair(float2 v) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1)
+    v = pair_add(v, make_float2(__shfl_xor_sync(0xffffffffu, v.x, d), __shfl_xor_sync(0xffffffffu, v.y, d)));
+  return v;
+}
+
+// The block's values added in a fixed tree, lanes then warps; the sum is
+// thread 0's.
 __device__ __forceinline__ float2 block_sum(float2 v, float2* sh) {
-  sh[threadIdx.x] = v;
+  v = warp_sum_pair(v);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
   __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if ((int)threadIdx.x < s) sh[threadIdx.x] = pair_add(sh[threadIdx.x], sh[threadIdx.x + s]);
-    __syncthreads();
-  }
-  const float2 r = sh[0];
-  __syncthreads();
-  return r;
+  if (threadIdx.x == 0)
+    for (int w = 1; w < kRedThreads / 32; ++w) v = pair_add(v, sh[w]);
+  __syncthreads();  // sh may be written again
+  return v;
 }
 
 struct ReduceJob {
@@ -76,10 +85,6 @@ struct ReduceJobs {
 
 // True in every thread of the block that finished a group last.
 __device__ __forceinline__ bool last_of_group(int* ticket, int splits) {
-  if (splits == 1) {  // the group's only block: no ticket to take
-    __syncthreads();  // its partial is visible to the block
-    return true;
-  }
   __shared__ int last;
   __threadfence();  // this block's partial is visible before its ticket
   __syncthreads();
@@ -104,6 +109,10 @@ __global__ void __launch_bounds__(kRedThreads) reduce_scalar(ReduceJobs js, int6
 #pragma unroll 8
   for (int64_t l = lo + threadIdx.x; l < hi; l += kRedThreads) acc += j.part[l];
   const float2 s = block_sum(make_float2(acc, 0.0f), sh);
+  if (S == 1) {  // the group's only block
+    if (threadIdx.x == 0) j.out[0] = pair_value(s);
+    return;
+  }
   if (threadIdx.x == 0) j.scratch[blockIdx.y] = s;
   if (!last_of_group(&j.tickets[0], S)) return;
   float2 t = make_float2(0.0f, 0.0f);
@@ -157,13 +166,28 @@ __global__ void __launch_bounds__(kRedThreads) reduce_per_channel(ReduceJobs js,
   const int64_t R = N / (C * HW);
   const int64_t runs = (B * R - s + S - 1) / S;  // runs j = s + q*S, q < runs
   float acc = 0.0f;  // a thread's elements in fp32, in order; the block's compensated
-  for (int64_t e = threadIdx.x; e < runs * HW; e += blockDim.x) {
-    const int64_t q = e / HW, h = e - q * HW;
-    const int64_t jr = s + q * S;
-    const int64_t b = jr / R, r = jr - b * R;
-    acc += j.part[b * N + (r * C + c) * HW + h];
+  if (runs * HW <= INT_MAX / 2 && B * R <= INT_MAX / 2) {  // the same in 32-bit divisions
+    const int n = (int)(runs * HW), hw = (int)HW, rr = (int)R;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < n; e += kRedThreads) {
+      const int q = e / hw, h = e - q * hw;
+      const int jr = (int)s + q * (int)S;
+      const int b = jr / rr, r = jr - b * rr;
+      acc += j.part[b * N + (r * C + c) * HW + h];
+    }
+  } else {
+    for (int64_t e = threadIdx.x; e < runs * HW; e += blockDim.x) {
+      const int64_t q = e / HW, h = e - q * HW;
+      const int64_t jr = s + q * S;
+      const int64_t b = jr / R, r = jr - b * R;
+      acc += j.part[b * N + (r * C + c) * HW + h];
+    }
   }
   const float2 v = block_sum(make_float2(acc, 0.0f), sh);
+  if (S == 1) {
+    if (threadIdx.x == 0) j.out[c] = pair_value(v);
+    return;
+  }
   if (threadIdx.x == 0) j.scratch[c * S + s] = v;
   if (!last_of_group(&j.tickets[c], (int)S)) return;
   if (threadIdx.x < 32) {  // lane l adds splits l, l + 32, ... in order, then a fixed tree
@@ -271,9 +295,11 @@ cudaError_t launch_param_reduce(const ParamReduce* p, int n, int64_t B, int64_t 
     if (e != cudaSuccess) return e;
   } else if (C > 0) {
     const int64_t R = N / (C * HW);
-    // about four blocks per SM in total, at least ~1k elements per block
+    // about four blocks per SM in total, at least 4096 elements per block: a
+    // channel of one block needs no second stage (its ticket and round trip
+    // through memory cost more than 16 elements a thread)
     int64_t S = ceil_div(608, C);
-    const int64_t by_size = ceil_div(B * R * HW, 1024);
+    const int64_t by_size = ceil_div(B * R * HW, 4096);
     if (S > by_size) S = by_size;
     if (S > B * R) S = B * R;
     if (S > scratch_len / C) S = scratch_len / C;
