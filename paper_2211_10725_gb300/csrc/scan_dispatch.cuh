@@ -23,9 +23,9 @@ inline bool few_lanes(int64_t L) {
   return device_info(&d) == cudaSuccess && L < 2048 * (int64_t)d.sms;
 }
 
-template <bool SYN, typename TI, typename TO, int RESET, bool REC, int VL, bool STRIPS>
-cudaError_t fwd_staged_vl(ScanArgs a, cudaStream_t st, bool* launched) {
-  const void* k = (const void*)scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, STRIPS>;
+template <bool SYN, typename TI, typename TO, int RESET, bool REC, int VL, bool STRIPS, bool CK>
+cudaError_t fwd_staged_ck(ScanArgs a, cudaStream_t st, bool* launched) {
+  const void* k = (const void*)scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, STRIPS, CK>;
   StagedPlan p;
   // a stage holds kFwdRows steps of the strip's input row; one CTA per SM
   // where it fits (the longer rows stream faster), two for short sequences
@@ -39,8 +39,14 @@ cudaError_t fwd_staged_vl(ScanArgs a, cudaStream_t st, bool* launched) {
   a.stage_bytes = p.stage_bytes;
   *launched = true;
   const int64_t grid = STRIPS && p.resident < p.grid ? p.resident : p.grid;
-  return launch_pdl(scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, STRIPS>, dim3((unsigned)grid),
+  return launch_pdl(scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, STRIPS, CK>, dim3((unsigned)grid),
                     dim3(p.threads), p.smem, st, a);
+}
+
+template <bool SYN, typename TI, typename TO, int RESET, bool REC, int VL, bool STRIPS>
+cudaError_t fwd_staged_vl(ScanArgs a, cudaStream_t st, bool* launched) {
+  return a.ckpt ? fwd_staged_ck<SYN, TI, TO, RESET, REC, VL, STRIPS, true>(a, st, launched)
+                : fwd_staged_ck<SYN, TI, TO, RESET, REC, VL, STRIPS, false>(a, st, launched);
 }
 
 // Short sequences (T <= 64) take 4 lanes a thread and CTAs that walk their

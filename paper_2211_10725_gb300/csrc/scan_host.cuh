@@ -191,6 +191,7 @@ inline void choose_parts(ScanArgs& a, const StagedPlan& p, int lanes) {
 // not instantiated.
 cudaError_t launch_scan_fwd(ScanArgs a, bool synaptic, int in_dt, int io_dt, bool staged,
                             cudaStream_t stream);
+cudaError_t launch_scan_fwd_synaptic(ScanArgs a, int in_dt, int io_dt, bool staged, cudaStream_t stream);
 cudaError_t launch_scan_bwd_leaky(ScanArgs a, bool recompute, int in_dt, int io_dt, bool staged,
                                   cudaStream_t stream);
 cudaError_t launch_scan_bwd_synaptic(ScanArgs a, bool recompute, int in_dt, int io_dt,

@@ -614,8 +614,13 @@ constexpr int kFwdRows = 8;
 // + gridDim.x, ... (else the grid has one CTA per strip): the ring runs on
 // across strips, so the next strip's rows arrive while the last steps of the
 // current one are computed.
+// CK: checkpoints may be due (the recompute mode).  Without them a whole
+// stage is kFwdRows steps with no test in them, and the spike bits are taken
+// from the packed spikes (with the tests, 28 instructions a neuron-step: the
+// recurrent neuron's forward at T = 100 over 64 x 4096 lanes in bf16 took 38
+// us, so 31; 23 us at 6.8 TB/s).
 template <bool SYN, typename TI, typename TO, int RESET, bool REC = false, int VL = kLanes<SYN>,
-          bool STRIPS = false>
+          bool STRIPS = false, bool CK = true>
 __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanArgs a) {
   constexpr int V = VL, NP = V / 2, R = kFwdRows;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -686,53 +691,115 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanA
         return;
       }
       const int nr = (int)min((int64_t)R, a.T - t0);
-      unsigned zbits[R];
-      if (active) {
-        const TI* st = my + pos.s * stage_elems;
+      if constexpr (!CK) {
+        uint32_t nibs = 0;  // V == 4: the thread's four spikes of step r at bit 4*r
+        auto step = [&](const TI* x_row, TO* spk_row, TO* mem_row, TO* syn_row, unsigned char* bit_byte,
+                        int r) {
+          float2 x[NP];
+          load_pairs<TI, NP>(x_row, x);
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          zbits[r] = 0;
-          if (r < nr) {
-            float2 x[NP];
-            load_pairs<TI, NP>(st + r * row_elems, x);
+          for (int k = 0; k < NP; ++k)
+            fwd_pair<SYN, RESET, REC ? 1 : 0>(a.reset, beta[k], negthr[k], third[k], x[k], u[k], z[k], in[k]);
+          if constexpr (sizeof(TO) == 2) {
+            uint32_t w[NP];
 #pragma unroll
-            for (int k = 0; k < NP; ++k)
-              fwd_pair<SYN, RESET, REC ? 1 : 0>(a.reset, beta[k], negthr[k], third[k], x[k], u[k],
-                                                z[k], in[k]);
+            for (int k = 0; k < NP; ++k) w[k] = Elem<TO>::from2(z[k].x, z[k].y);
+            if constexpr (V == 8) *reinterpret_cast<uint4*>(spk_row) = make_uint4(w[0], w[1], w[2], w[3]);
+            else *reinterpret_cast<uint2*>(spk_row) = make_uint2(w[0], w[1]);
             if (bits) {
+              // one set bit of 1.0's exponent per half: bf16 0x3F80, fp16 0x3C00
+              constexpr uint32_t one = std::is_same<TO, __half>::value ? 0x04000400u : 0x00800080u;
+              constexpr int at = std::is_same<TO, __half>::value ? 10 : 7;
+              uint32_t t = 0;
 #pragma unroll
-              for (int k = 0; k < NP; ++k) {
-                zbits[r] |= ((z[k].x != 0.0f) ? 1u : 0u) << (2 * k);
-                zbits[r] |= ((z[k].y != 0.0f) ? 1u : 0u) << (2 * k + 1);
-              }
+              for (int k = 0; k < NP; ++k) t |= ((w[k] & one) >> at) << (2 * k);
+              t = (t | (t >> 15)) & ((1u << V) - 1u);
+              if constexpr (V == 8) *bit_byte = (unsigned char)t;
+              else nibs |= t << (4 * r);
             }
-            store_pairs<TO, NP>(spk + r * a.L, z);
-            if (mem) store_pairs<TO, NP>(mem + r * a.L, u);
-            if (SYN && syn) store_pairs<TO, NP>(syn + r * a.L, in);
-            if (++kk == a.K) {
-              kk = 0;
-              if (ck && t0 + r + 1 < a.T) {
-                store_pairs<float, NP>(ck, u);
-                if (SYN) store_pairs<float, NP>(ck + a.L, in);
-                ck += ck_stride;
+          } else {
+            store_pairs<TO, NP>(spk_row, z);
+          }
+          if (mem) store_pairs<TO, NP>(mem_row, u);
+          if (SYN && syn) store_pairs<TO, NP>(syn_row, in);
+        };
+        if (active) {
+          const TI* st = my + pos.s * stage_elems;
+          const int64_t L = a.L;
+          if (nr == R) {
+#pragma unroll
+            for (int r = 0; r < R; ++r)
+              step(st + r * row_elems, spk + r * L, mem + r * L, syn + r * L, bits + r * a.bits_row, r);
+          } else {
+#pragma unroll 1
+            for (int r = 0; r < nr; ++r)
+              step(st + r * row_elems, spk + r * L, mem + r * L, syn + r * L, bits + r * a.bits_row, r);
+          }
+        }
+        if (bits) {
+          if constexpr (V == 4) {
+            // a byte's halves sit in neighbouring threads: the even one stores
+            // the stage's first four steps, the odd one the others
+            const uint32_t other = __shfl_xor_sync(0xffffffffu, nibs, 1);
+            const int odd = c & 1;
+            const uint32_t lo = (odd ? other : nibs) >> (16 * odd), hi = (odd ? nibs : other) >> (16 * odd);
+#pragma unroll
+            for (int k = 0; k < R / 2; ++k)
+              if (active && k + odd * (R / 2) < nr)
+                bits[(k + odd * (R / 2)) * a.bits_row] =
+                    (unsigned char)(((lo >> (4 * k)) & 15u) | (((hi >> (4 * k)) & 15u) << 4));
+          }
+          bits += R * a.bits_row;
+        }
+      } else {
+        unsigned zbits[R];
+        if (active) {
+          const TI* st = my + pos.s * stage_elems;
+#pragma unroll
+          for (int r = 0; r < R; ++r) {
+            zbits[r] = 0;
+            if (r < nr) {
+              float2 x[NP];
+              load_pairs<TI, NP>(st + r * row_elems, x);
+#pragma unroll
+              for (int k = 0; k < NP; ++k)
+                fwd_pair<SYN, RESET, REC ? 1 : 0>(a.reset, beta[k], negthr[k], third[k], x[k], u[k],
+                                                  z[k], in[k]);
+              if (bits) {
+#pragma unroll
+                for (int k = 0; k < NP; ++k) {
+                  zbits[r] |= ((z[k].x != 0.0f) ? 1u : 0u) << (2 * k);
+                  zbits[r] |= ((z[k].y != 0.0f) ? 1u : 0u) << (2 * k + 1);
+                }
+              }
+              store_pairs<TO, NP>(spk + r * a.L, z);
+              if (mem) store_pairs<TO, NP>(mem + r * a.L, u);
+              if (SYN && syn) store_pairs<TO, NP>(syn + r * a.L, in);
+              if (++kk == a.K) {
+                kk = 0;
+                if (ck && t0 + r + 1 < a.T) {
+                  store_pairs<float, NP>(ck, u);
+                  if (SYN) store_pairs<float, NP>(ck + a.L, in);
+                  ck += ck_stride;
+                }
               }
             }
           }
         }
-      }
-      if (bits) {
+        if (bits) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          if (r < nr) {
-            if (V == 4) {
-              const unsigned hi = __shfl_down_sync(0xffffffffu, zbits[r], 1);
-              if (active && !(c & 1)) bits[r * a.bits_row] = (unsigned char)(zbits[r] | (hi << 4));
-            } else if (active) {
-              bits[r * a.bits_row] = (unsigned char)zbits[r];
+          for (int r = 0; r < R; ++r) {
+            if (r < nr) {
+              if (V == 4) {
+                const unsigned hi = __shfl_down_sync(0xffffffffu, zbits[r], 1);
+                if (active && !(c & 1)) bits[r * a.bits_row] = (unsigned char)(zbits[r] | (hi << 4));
+              } else if (active) {
+                bits[r * a.bits_row] = (unsigned char)zbits[r];
+              }
             }
           }
+          bits += R * a.bits_row;
         }
-        bits += R * a.bits_row;
       }
       release_stage(empty, pos.s, lid);
       pos.next(S);
