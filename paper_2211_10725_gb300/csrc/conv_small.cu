@@ -8,10 +8,10 @@
 //             k = (ky*KW + kx)*Cin + c, fp32 fused multiply-adds in k order
 //   weight    dW[o, k] = sum over (m, oy, ox) of dI[m, oy, ox, o] *
 //   gradient  X[m, oy+ky, ox+kx, c]; block b sums images b, b + G, ... in
-//             order, lanes add their pixels in order, and the warp trees
-//             and the final sum over the G block partials (strided lane sums,
-//             then a shuffle tree) run in a fixed order, so the result is
-//             the same on every call.
+//             order, and the sums within a block and over the G block
+//             partials run in a fixed order, so the result is the same on
+//             every call.  One input channel with 8 or 16 outputs and an
+//             even output width runs on the tensor cores.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 

@@ -3,6 +3,8 @@
 //   D[M, N] = A[M, K] * B[N, K]^T,   A, B bf16 row-major (K contiguous),
 // fp32 accumulation in tensor memory, fp32 or bf16 output.
 //
+// Products that the operands' way into the SMs would bound run on pairs of
+// CTAs (gemm_pair_tcgen05 below); the others on single CTAs, as follows.
 // Persistent CTAs (one per SM) take 128 x BN tiles (BN up to 256) in turn.  Warp 0 (one
 // thread) streams 128x64 and BNx64 operand tiles into a shared-memory ring
 // with TMA (128-byte swizzle), 8, 6 or 4 stages deep for BN = 64, 128, 256
@@ -32,7 +34,7 @@
 // Split K: a product whose few output tiles each sum a long K (the weight
 // gradient of a convolution sums over every patch row) runs as tiles x S
 // work items, item (tile, s) summing k-blocks [s*nk/S, (s+1)*nk/S) into
-// partial output s; a second kernel adds the S partials in split order, so
+// partial output s; a second kernel adds the S partials in a fixed order, so
 // the result does not depend on which CTA ran which item.  Weight gradients
 // of wide layers use 128 x 256 tiles (four 64-column MN-major B boxes) and
 // splits, which cuts the re-reads of dI across output columns.

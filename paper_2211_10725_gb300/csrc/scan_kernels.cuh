@@ -3,12 +3,13 @@
 //
 // Layout: every [T, B, N] tensor is t-major, so the L = B*N lanes of one step
 // are contiguous.  A lane is independent of every other lane and sequential
-// in t: each thread owns 8 (Leaky) or 4 (Synaptic) consecutive lanes and keeps their state (u, i,
+// in t: each thread owns 8 or 4 consecutive lanes and keeps their state (u, i,
 // z and, backward, the adjoints) in registers for the whole scan.
 //
-// Staged kernels (the fast path): a CTA owns a contiguous strip of lanes.
-// One producer thread streams the strip's row of every input tensor, step by
-// step, into a ring of shared-memory stages with 1-D bulk copies (TMA,
+// Staged kernels (the fast path): a CTA owns a contiguous strip of lanes, or
+// walks several (short sequences).
+// One producer thread streams the strip's row of every input tensor, a few
+// steps at a time, into a ring of shared-memory stages with 1-D bulk copies (TMA,
 // cp.async.bulk) completing on a "full" mbarrier per stage; the consumer
 // warps wait on it, read their lanes, compute and store the step, and only
 // then release the stage on its "empty" mbarrier.  The ring depth, not the
