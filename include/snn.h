@@ -498,7 +498,8 @@ snn_status_t snn_conv2d_small_dw_nhwc(int64_t M, int64_t H, int64_t W, int64_t C
  *   pool     bf16 [T*B, Ho/2, Wo/2, Cout] (out) and idx uint8 (out): the
  *            pooled spikes and positions, or both NULL
  * Cin = 1, KH = KW of 3 or 5, Cout = 16, Ho and Wo even, H*W a multiple
- * of 8 and at most 8192; SNN_ERR_UNSUPPORTED otherwise.  Initial state zero.
+ * of 8 and at most 8192, W at most 190 (two buffers of 8 steps' image rows in
+ * shared memory); SNN_ERR_UNSUPPORTED otherwise.  Initial state zero.
  */
 snn_status_t snn_conv2d_small_leaky_fwd_nhwc(const snn_scan_desc* desc, int64_t H, int64_t W,
                                              int64_t Cin, int64_t Cout, int64_t KH, int64_t KW,

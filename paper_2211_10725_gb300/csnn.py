@@ -81,9 +81,11 @@ class ConvSNN:
         self.direct = [direct_first and g0[4] * g0[4] * g0[2] <= 32 and g0[3] <= 16
                        and g0[0] * g0[1] * g0[2] <= 8192] + [False] * (len(self.geo) - 1)
         # ... and, with the traces stored, in one kernel with its scan and pooling
-        # (the shapes snn_conv2d_small_leaky_fwd_nhwc takes)
+        # (the shapes snn_conv2d_small_leaky_fwd_nhwc takes; it stages 8 steps of up
+        # to 8 image rows twice in 48 KB, which rows of at most 190 pixels always fit)
         self.direct_scan = [self.fused and d and g[2] == 1 and g[4] in (3, 5) and g[3] == 16
                             and g[5] % 2 == 0 and g[6] % 2 == 0 and g[0] * g[1] % 8 == 0
+                            and g[1] <= 190
                             for d, g in zip(self.direct, self.geo)]
         self.n_out = _pad8(w.n_classes)
 

@@ -136,7 +136,7 @@ def _check(status: int, where: str):
 
 
 def _ptr(t) -> Optional[int]:
-    if t is None or type(t) is int:
+    if t is None or isinstance(t, int):
         return t
     return t.data_ptr()
 

@@ -62,6 +62,19 @@ def test_population_network_keeps_the_unfused_backward_at_one_step():
     assert net.layers[-1].w.N == 504   # 10 classes x 50, padded to a multiple of 8
 
 
+@pytest.mark.parametrize("H,Wd,one_kernel", [(28, 28, True), (40, 190, True), (32, 192, False),
+                                             (32, 256, False)])
+def test_first_layer_of_wide_maps_keeps_its_separate_kernels(H, Wd, one_kernel):
+    """Image rows too wide to stage run as convolution, scan and pooling."""
+    w = W.CSNN_C4.scaled(T=2, B=2, H=H, W=Wd)
+    inp = W.make_conv_inputs(w)
+    net = ConvSNN(w, inp["convs"], inp["Wfc"], device="cpu", save="fused")
+    names = _names(net)
+    assert net.direct[0] and names[0] == "conv_fwd0"
+    assert ("scan_fwd0" not in names and "pool_fwd0" not in names) == one_kernel
+    assert (net.I[0] is None) == one_kernel
+
+
 @pytest.mark.parametrize("save", ["recompute", "mem", "fused"])
 def test_conv_network_launch_order(save):
     w = W.CSNN_C4
