@@ -572,7 +572,8 @@ __device__ __forceinline__ void initial_state(const ScanArgs& a, int64_t l, cons
 
 // One parameter's gradient partials of a consumer warp, in the layout the
 // launch chose; every lane of the warp calls it (an inactive thread adds
-// zeros).  gw: the warp's index among the launch's consumer warps.
+// zeros).  gw: the warp's index among the launch's consumer warps.  Tens of
+// terms are added in fp32, more in compensated fp32.
 template <int V>
 __device__ __forceinline__ void store_partials(const ScanArgs& a, float* part, int kind, float (&v)[V],
                                                int64_t l, bool active, int64_t gw, int lid) {
@@ -583,7 +584,7 @@ __device__ __forceinline__ void store_partials(const ScanArgs& a, float* part, i
 #pragma unroll
   for (int k = 0; k < V; ++k)
     if (!active) v[k] = 0.0f;
-  if (kind == PART_CHANNELS) {  // threads C / V apart hold the same channels
+  if (kind == PART_CHANNELS) {  // threads C / V apart hold the same channels: at most 16 terms
     const int period = (int)a.C / V;
     for (int d = period; d < 32; d <<= 1)
 #pragma unroll
@@ -594,13 +595,16 @@ __device__ __forceinline__ void store_partials(const ScanArgs& a, float* part, i
   float s = 0.0f;
 #pragma unroll
   for (int k = 0; k < V; k += 2) s += v[k] + v[k + 1];
-  const int group = kind == PART_WARP ? 32 : a.part_q / V;  // threads that add up
-  for (int d = 1; d < group; d <<= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-  if (kind == PART_WARP) {
-    if (lid == 0) part[gw] = s;
-  } else if (active && (lid & (group - 1)) == 0) {
-    part[l / a.part_q] = s;
+  if (kind == PART_WARP) {  // up to 256 terms: compensated across the lanes
+    float2 p = make_float2(s, 0.0f);
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) p = pair_add(p, shfl_xor_pair(p, d));
+    if (lid == 0) part[gw] = pair_value(p);
+    return;
   }
+  const int group = a.part_q / V;  // threads that add up: at most 32 terms
+  for (int d = 1; d < group; d <<= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
+  if (active && (lid & (group - 1)) == 0) part[l / a.part_q] = s;
 }
 
 // ---------------------------------------------------------------------------

@@ -231,4 +231,30 @@ __device__ __forceinline__ void storev(T* p, const float* v) {
   else Elem<T>::store4(p, v);
 }
 
+// ---- compensated sums ------------------------------------------------------
+
+// (sum, error) += x: the rounding error of the addition kept in .y
+// (two-sum; every operation rounded to nearest, none fused).
+__device__ __forceinline__ float2 two_add(float2 a, float x) {
+  const float s = __fadd_rn(a.x, x);
+  const float z = __fadd_rn(s, -a.x);
+  const float e = __fadd_rn(__fadd_rn(a.x, -__fadd_rn(s, -z)), __fadd_rn(x, -z));
+  return make_float2(s, __fadd_rn(a.y, e));
+}
+// (sum, error) += (sum', error')
+__device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
+  a = two_add(a, b.x);
+  a.y = __fadd_rn(a.y, b.y);
+  return a;
+}
+// The pair's value; a non-finite sum is returned as it is (its error term
+// is NaN once an infinity entered the sum).
+__device__ __forceinline__ float pair_value(float2 a) {
+  return isfinite(a.x) ? __fadd_rn(a.x, a.y) : a.x;
+}
+
+__device__ __forceinline__ float2 shfl_xor_pair(float2 v, int d) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, v.x, d), __shfl_xor_sync(0xffffffffu, v.y, d));
+}
+
 }  // namespace snn
