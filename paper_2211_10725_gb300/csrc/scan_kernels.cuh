@@ -1303,33 +1303,36 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_bwd_staged(const ScanA
 // ---------------------------------------------------------------------------
 // Plain kernels: one lane per thread, direct loads, any shape.
 // The recurrence needs the rows one after another, but their loads depend on
-// nothing, so each thread keeps kPlainAhead to 2*kPlainAhead steps' loads in
-// flight: with one step's load on the chain at a time a step cost a memory
+// nothing, so each thread keeps 16 to 32 steps' loads in flight (8 to 16 in
+// a checkpoint segment): with one step's load on the chain at a time a step cost a memory
 // latency.  T = 75, 33 x 1001 lanes in half precision, both passes: 52 us;
-// with the loads ahead 33, and with the modes compiled in and pointers that
-// walk instead of 64-bit address products 25 (4 us at 6.7 TB/s: the lanes
-// are one or two warps a scheduler, so a step's instructions bound it).
+// with 8 to 16 steps' loads ahead 33, with the modes compiled in and pointers
+// that walk instead of 64-bit address products 25.2, and with 16 to 32 steps
+// 24.5 (4 us at 6.7 TB/s: the lanes are one or two warps a scheduler, so a
+// step's instructions bound it).  Segments of 12 steps took 44.6 us with 16
+// ahead, 37.5 with 8.
 // ---------------------------------------------------------------------------
 
-constexpr int kPlainAhead = 8;
+constexpr int kPlainAhead = 16;    // whole sequences
+constexpr int kPlainAheadSeg = 8;  // checkpoint segments, most of them shorter than 16 steps
 
-// step(i, item) for i = 0 .. n-1 in order, item = load(i) issued kPlainAhead
-// to 2*kPlainAhead steps before it is used.
-template <typename Item, typename Load, typename Step>
+// step(i, item) for i = 0 .. n-1 in order, item = load(i) issued A to 2*A
+// steps before it is used.
+template <typename Item, int A, typename Load, typename Step>
 __device__ __forceinline__ void plain_steps(int64_t n, Load load, Step step) {
-  Item cur[kPlainAhead], next[kPlainAhead];
+  Item cur[A], next[A];
 #pragma unroll
-  for (int k = 0; k < kPlainAhead; ++k)
+  for (int k = 0; k < A; ++k)
     if (k < n) cur[k] = load(k);
-  for (int64_t i = 0; i < n; i += kPlainAhead) {
+  for (int64_t i = 0; i < n; i += A) {
 #pragma unroll
-    for (int k = 0; k < kPlainAhead; ++k)
-      if (i + kPlainAhead + k < n) next[k] = load(i + kPlainAhead + k);
+    for (int k = 0; k < A; ++k)
+      if (i + A + k < n) next[k] = load(i + A + k);
 #pragma unroll
-    for (int k = 0; k < kPlainAhead; ++k)
+    for (int k = 0; k < A; ++k)
       if (i + k < n) step(i + k, cur[k]);
 #pragma unroll
-    for (int k = 0; k < kPlainAhead; ++k) cur[k] = next[k];
+    for (int k = 0; k < A; ++k) cur[k] = next[k];
   }
 }
 
@@ -1352,7 +1355,7 @@ __global__ void __launch_bounds__(128) scan_fwd_plain(const ScanArgs a) {
   const int64_t ckpt_stride = SYN ? 2 * a.L : a.L;
   int kk = a.nseg > 0 ? seg_phase0(a) : 0;
   float* cp = a.ckpt ? a.ckpt + l : nullptr;
-  plain_steps<TI>(
+  plain_steps<TI, kPlainAhead>(
       a.T,
       [&](int64_t) {
         const TI x = *I;
@@ -1415,7 +1418,7 @@ __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
     struct Item {
       TO g, u, z, i, m;
     };
-    plain_steps<Item>(
+    plain_steps<Item, kPlainAhead>(
         a.T,
         [&](int64_t) {
           Item it;
@@ -1460,14 +1463,14 @@ __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
         i = s0;
         z = have_mem0 && (m0 > thr);
       }
-      plain_steps<TI>(
+      plain_steps<TI, kPlainAheadSeg>(
           t1 - t0, [&](int64_t j) { return I[(t0 + j) * a.L]; },
           [&](int64_t j, const TI& x) {
             fwd_step<SYN, RESET, REC>(a.reset, beta, thr, alpha, Elem<TI>::load1(&x), u, z, i, a.rec != 0);
             su[j * blockDim.x] = u;
             if (SYN) si[j * blockDim.x] = i;
           });
-      plain_steps<Item>(
+      plain_steps<Item, kPlainAheadSeg>(
           t1 - t0,
           [&](int64_t j) {
             const int64_t off = (t1 - 1 - j) * a.L;
