@@ -244,9 +244,17 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
         // to 0; the staged value of (t, lane) is dL/dz_t.  The stored trace
         // comes in chunks of kBwdChunk steps, the next chunk's loads issued
         // before the current chunk is stepped, so a lane waits for memory
-        // about once rather than once per step.
+        // about once rather than once per step.  A whole chunk's steps are
+        // straight-line code behind its eight gradients (a step's shared
+        // read stood behind the step before's store), and a warp whose lanes
+        // are wholly past the tile has none (T = 100 leaves 64 lanes a
+        // tile): T = 25, B = 128, 1000 x 1000 20.1 -> 19.3 us, T = 40 40.6
+        // -> 30.8, T = 100 and B = 256 256 -> 193.  The same in the forward
+        // scan was slower (T = 100, B = 64: 41 -> 55 us; the idle warps'
+        // skip alone 41 -> 40 there, but 17.2 -> 18.3 for 104 inputs at T =
+        // 25, B = 256).
         const int64_t RN = (int64_t)f.R * f.N;
-        for (int g0 = 0; g0 < lanes; g0 += kScanThreads) {
+        for (int g0 = 0; g0 + (e & ~31) < lanes; g0 += kScanThreads) {
           const int j = g0 + e;
           const int jj = j < lanes ? j : 0;  // lanes past the tile read row 0
           const int sr = jj / BN, n = jj - (jj / BN) * BN;
@@ -275,16 +283,25 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
           __nv_bfloat16 ucur[kBwdChunk], unext[kBwdChunk];
           uint32_t zcur, znext = 0;
           load_chunk(f.T - 1, ucur, zcur);
+          auto step = [&](int c, int ts, float gs) {
+            const float du =
+                bwd_step<false, RESET, SG, 0>(f.sa, beta, thr, 0.0f, ts + 1 < f.T, __bfloat162float(ucur[c]),
+                                              ((zcur >> c) & 1u) != 0, 0.0f, gs, 0.0f, 0.0f, st);
+            if (ok) f.gI[(int64_t)ts * RN + o] = __float2bfloat16_rn(du);
+          };
+          const int gstep = f.BS * SP;
           for (int tc = f.T - 1; tc >= 0; tc -= kBwdChunk) {
             if (tc - kBwdChunk >= 0) load_chunk(tc - kBwdChunk, unext, znext);
+            if (tc >= kBwdChunk - 1) {  // a whole chunk: its gradients first, then no test per step
+              float gs[kBwdChunk];
 #pragma unroll
-            for (int c = 0; c < kBwdChunk; ++c) {
-              const int ts = tc - c;
-              if (ts < 0) break;
-              const float du =
-                  bwd_step<false, RESET, SG>(f.sa, beta, thr, 0.0f, ts + 1 < f.T, __bfloat162float(ucur[c]),
-                                             ((zcur >> c) & 1u) != 0, 0.0f, gsp[ts * f.BS * SP], 0.0f, 0.0f, st);
-              if (ok) f.gI[(int64_t)ts * RN + o] = __float2bfloat16_rn(du);
+              for (int c = 0; c < kBwdChunk; ++c) gs[c] = gsp[(tc - c) * gstep];
+#pragma unroll
+              for (int c = 0; c < kBwdChunk; ++c) step(c, tc - c, gs[c]);
+            } else {
+#pragma unroll
+              for (int c = 0; c < kBwdChunk; ++c)
+                if (tc - c >= 0) step(c, tc - c, gsp[(tc - c) * gstep]);
             }
 #pragma unroll
             for (int c = 0; c < kBwdChunk; ++c) ucur[c] = unext[c];
