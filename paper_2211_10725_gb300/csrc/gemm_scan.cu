@@ -24,12 +24,6 @@
 // in reverse time with the scan kernels' bwd_step, from its stored bf16
 // trace and spike bits, writing its dL/dI.  The spike gradient is never
 // rounded or written.
-//
-// CL = 2: clusters of two CTAs on neighbouring column tiles of one row tile
-// take turns to load A's box for both (TMA multicast).  A stage's `empty`
-// barrier collects both CTAs' commits, so whoever fills it next knows that
-// both have used it; each CTA's `full` barrier counts its own bytes,
-// whichever CTA asked for them.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -84,7 +78,7 @@ __device__ __forceinline__ void epi_barrier() {
   asm volatile("bar.sync 1, %0;" ::"n"(kScanThreads) : "memory");
 }
 
-template <int BN, int RESET, bool BWD = false, int SG = 0, int CL = 1>
+template <int BN, int RESET, bool BWD = false, int SG = 0>
 __global__ void __launch_bounds__(kFusedThreads, 2)
     gemm_leaky_tcgen05(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                        const FusedArgs f) {
@@ -109,18 +103,14 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
   int* epi_ok = reinterpret_cast<int*>(tmem_slot + 1);  // [4] per epilogue warp: its wait succeeded
   const int warp = threadIdx.x >> 5, lid = threadIdx.x & 31;
   const int nk = (f.K + BK - 1) / BK;
-  // work items: CL neighbouring column tiles of a row tile, one per CTA
-  const int rank = CL > 1 ? (int)cluster_rank() : 0;
-  const int item0 = (int)blockIdx.x / CL, item_step = (int)gridDim.x / CL;
-  const int groups_n = ((f.N + BN - 1) / BN + CL - 1) / CL;
-  const int items = groups_n * ((f.R + f.BS - 1) / f.BS);
-  constexpr uint16_t kAll = (uint16_t)((1u << CL) - 1u);
+  const int tiles_n = (f.N + BN - 1) / BN;
+  const int tiles = tiles_n * ((f.R + f.BS - 1) / f.BS);
   const uint32_t a_tx = (uint32_t)(f.BS * f.T * 128);  // bytes of one A box
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kFusedStages; ++s) {
       mbar_init(&full[s], 1);
-      mbar_init(&empty[s], CL);
+      mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(&acc_full[b], 1);
@@ -131,7 +121,6 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
   if (warp == 1) tmem_alloc(tmem_slot, TCOLS);
   tc_fence_before();
   __syncthreads();
-  if (CL > 1) cluster_barrier();  // every CTA's barriers are initialised
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   grid_dep_wait();
@@ -140,8 +129,8 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
     if (lid == 0) {
       int64_t n_issued = 0;
       bool ok = true;
-      for (int t = item0; t < items && ok; t += item_step) {
-        const int r0 = (t / groups_n) * f.BS, n0 = ((t % groups_n) * CL + rank) * BN;
+      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x) {
+        const int r0 = (t / tiles_n) * f.BS, n0 = (t % tiles_n) * BN;
         for (int kb = 0; kb < nk; ++kb, ++n_issued) {
           const int s = (int)(n_issued % kFusedStages);
           if (n_issued >= kFusedStages &&
@@ -151,10 +140,7 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
             break;
           }
           mbar_arrive_expect_tx(&full[s], a_tx + B_BYTES);
-          if (CL == 1)
-            tma_load_3d(sA + s * A_BYTES, &ta, kb * BK, r0, 0, &full[s]);
-          else if ((int)(n_issued % CL) == rank)  // the cluster's CTAs take turns to load A for all
-            tma_load_3d_multicast(sA + s * A_BYTES, &ta, kb * BK, r0, 0, &full[s], kAll);
+          tma_load_3d(sA + s * A_BYTES, &ta, kb * BK, r0, 0, &full[s]);
           if constexpr (BWD) {
 #pragma unroll
             for (int j = 0; j < BN / 64; ++j)
@@ -176,7 +162,7 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
       int64_t n_used = 0;
       bool ok = true;
       int i = 0;
-      for (int t = item0; t < items && ok; t += item_step, ++i) {
+      for (int t = blockIdx.x; t < tiles && ok; t += gridDim.x, ++i) {
         const int b = i & 1;
         if (i >= 2 && !mbar_wait_poll(&acc_empty[b], (uint32_t)(((i >> 1) - 1) & 1), f.wait_ns)) {
           record_status(f.status, kStatusTimeout);
@@ -197,8 +183,7 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
 #pragma unroll
           for (int kk = 0; kk < BK / 16; ++kk)
             tc_mma(acc, da + (uint64_t)(2 * kk), db + stepB * kk, idesc, (kb | kk) != 0 ? 1u : 0u);
-          if (CL == 1) tc_commit(&empty[s]);
-          else tc_commit_multicast(&empty[s], kAll);  // this CTA has used the stage, for whoever fills it
+          tc_commit(&empty[s]);
         }
         if (ok) tc_commit(&acc_full[b]);
       }
@@ -209,11 +194,11 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
     const int e = threadIdx.x - 64;  // 0..kScanThreads-1 among the scan threads
     const int lanes = f.BS * BN;
     int i = 0;
-    for (int t = item0; t < items; t += item_step, ++i) {
+    for (int t = blockIdx.x; t < tiles; t += gridDim.x, ++i) {
       const int b = i & 1;
       const bool waited =
           drains ? warp_wait_uniform(&acc_full[b], (uint32_t)((i >> 1) & 1), f.wait_ns) : true;
-      const int r0 = (t / groups_n) * f.BS, n0 = ((t % groups_n) * CL + rank) * BN;
+      const int r0 = (t / tiles_n) * f.BS, n0 = (t % tiles_n) * BN;
       if (drains && waited) {
         tc_fence_after();
         // accumulator -> shared memory: row = TMEM lane = (t, r) of the tile
@@ -369,35 +354,16 @@ __global__ void __launch_bounds__(kFusedThreads, 2)
   }
   tc_fence_before();
   __syncthreads();
-  if (CL > 1) cluster_barrier();  // no CTA leaves while another may still write to it or signal it
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, TCOLS);
   }
 }
 
-// Pairs of CTAs that share a row tile (CL = 2): where the operands' rows are
-// no whole cache lines.  A 128-byte row of a box then takes two lines, and
-// the loads are bound by lines rather than bytes; a pair requests 64 + 64
-// rows a k-block per CTA instead of 128 + 64.  T = 25, B = 128, 1000 inputs
-// and outputs: forward 20.1 -> 18.2 us, backward 22.5 -> 20.4; 3064 inputs
-// 47.1 -> 39.7.  Not with whole lines (1024: 15.7 -> 16.7, the pair runs in
-// step and the SM's intake of bytes is the bound), nor, backward, with W's
-// rows alone whole (15.3 -> 15.8), nor for fewer than 16 k-blocks (784
-// inputs: 14.7 -> 15.5), less than a tile per SM (B = 32: 9.6 -> 10.4) or
-// one row r per tile, whose scan is the bound (T = 100, B = 256: 128.0 ->
-// 129.4).  Clusters of four were slower in every case.
-bool shares_rows(const FusedArgs& f, int bn, bool bwd) {
-  DeviceInfo d;
-  const int64_t tiles_n = (f.N + bn - 1) / bn;
-  return f.K % 64 != 0 && (!bwd || f.N % 64 != 0) && tiles_n % 2 == 0 && (f.K + BK - 1) / BK >= 16 &&
-         f.BS >= 2 && device_info(&d) == cudaSuccess && tiles_n * ((f.R + f.BS - 1) / f.BS) > d.sms;
-}
-
-template <int BN, int RESET, bool BWD, int SG, int CL>
-cudaError_t launch_fused_cl(const CUtensorMap& ta, const CUtensorMap& tb, const FusedArgs& f,
-                            cudaStream_t st) {
-  const void* k = (const void*)gemm_leaky_tcgen05<BN, RESET, BWD, SG, CL>;
+template <int BN, int RESET, bool BWD = false, int SG = 0>
+cudaError_t launch_fused(const CUtensorMap& ta, const CUtensorMap& tb, const FusedArgs& f,
+                         cudaStream_t st) {
+  const void* k = (const void*)gemm_leaky_tcgen05<BN, RESET, BWD, SG>;
   const cudaError_t attr = ensure_smem(k, fused_smem_bytes<BN>());
   if (attr != cudaSuccess) return attr;
   int dev = 0, sms = 152, per_sm = 1;
@@ -409,19 +375,10 @@ cudaError_t launch_fused_cl(const CUtensorMap& ta, const CUtensorMap& tb, const 
     per_sm = 1;
   if (fused_smem_bytes<BN>() * 2 <= 220 * 1024) per_sm = per_sm < 2 ? 2 : per_sm;  // fits twice
   const int64_t slots = (int64_t)sms * (per_sm > 2 ? 2 : per_sm);
-  const int64_t items = (((f.N + BN - 1) / BN + CL - 1) / CL) * (int64_t)((f.R + f.BS - 1) / f.BS);
-  const int64_t clusters = items < slots / CL ? items : slots / CL;
-  return launch_pdl_cluster(CL > 1 ? CL : 0, gemm_leaky_tcgen05<BN, RESET, BWD, SG, CL>,
-                            dim3((unsigned)(clusters * CL)), dim3(kFusedThreads), fused_smem_bytes<BN>(), st, ta,
-                            tb, f);
-}
-
-template <int BN, int RESET, bool BWD = false, int SG = 0>
-cudaError_t launch_fused(const CUtensorMap& ta, const CUtensorMap& tb, const FusedArgs& f,
-                         cudaStream_t st) {
-  if constexpr (BN >= 64)
-    if (shares_rows(f, BN, BWD)) return launch_fused_cl<BN, RESET, BWD, SG, 2>(ta, tb, f, st);
-  return launch_fused_cl<BN, RESET, BWD, SG, 1>(ta, tb, f, st);
+  const int64_t tiles = (int64_t)((f.N + BN - 1) / BN) * ((f.R + f.BS - 1) / f.BS);
+  const unsigned grid = (unsigned)(tiles < slots ? tiles : slots);
+  return launch_pdl(gemm_leaky_tcgen05<BN, RESET, BWD, SG>, dim3(grid), dim3(kFusedThreads),
+                    fused_smem_bytes<BN>(), st, ta, tb, f);
 }
 
 template <int BN, int SG>

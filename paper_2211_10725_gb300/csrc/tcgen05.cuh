@@ -171,25 +171,6 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint64_t* bar, uint32_t rank
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr(bar, rank))
                : "memory");
 }
-// 3-D tile load into the same place of every CTA in `mask` (cluster ranks),
-// completing on the same barrier of each.
-__device__ __forceinline__ void tma_load_3d_multicast(void* dst, const CUtensorMap* map, int x, int y, int z,
-                                                      uint64_t* bar, uint16_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
-      "[%1, {%2, %3, %4}], [%5], %6;" ::"r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar)), "h"(mask)
-      : "memory");
-}
-// Arrive on `bar` of every CTA in `mask` once this thread's (single-CTA) MMAs
-// so far are done.
-__device__ __forceinline__ void tc_commit_multicast(uint64_t* bar, uint16_t mask) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-          smem_u32(bar)),
-      "h"(mask)
-      : "memory");
-}
 // M = 256 over the pair: each CTA's shared memory holds 128 rows of A and
 // half of B's columns, its tensor memory 128 rows of D.
 __device__ __forceinline__ void tc_mma_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc,
