@@ -429,11 +429,19 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
         }
       }
-      // every copy has landed before the CTAs may exit: the leader's barriers
-      // count both CTAs' copies
+      // Before the CTAs may exit, every copy has landed (the leader's `full`
+      // barriers count both CTAs') and the leader's last commit has arrived on
+      // each stage's `empty` in both CTAs: those arrivals are not ordered with
+      // the one on `acc_full` that lets the epilogue finish, nor with the
+      // cluster barrier.
+      const int64_t last = n_issued > kStages ? n_issued - kStages : 0;
+      bool drained = true;
       if (rank == 0)
-        for (int64_t j = n_issued > kStages ? n_issued - kStages : 0; j < n_issued; ++j)
-          mbar_wait_bounded(&full[j % kStages], (uint32_t)((j / kStages) & 1), kDrainWaitNs);
+        for (int64_t j = last; j < n_issued && drained; ++j)
+          drained = mbar_wait_bounded(&full[j % kStages], (uint32_t)((j / kStages) & 1), kDrainWaitNs);
+      drained = true;
+      for (int64_t j = last; j < n_issued && drained; ++j)
+        drained = mbar_wait_bounded(&empty[j % kStages], (uint32_t)((j / kStages) & 1), kDrainWaitNs);
     }
   } else if (warp == 1) {
     if (rank == 0 && lid == 0) {
@@ -496,7 +504,9 @@ __global__ void __launch_bounds__(kThreads, 1)
   }
   tc_fence_before();
   __syncthreads();
-  cluster_barrier();  // neither CTA leaves while the other may still signal it
+  // neither CTA leaves before the other has read and signalled its last; the
+  // asynchronous arrivals were waited for above
+  cluster_barrier();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc_pair(tmem, TCOLS);

@@ -17,3 +17,24 @@ def test_no_load_writes_another_blocks_shared_memory():
                 loads += 1
                 assert "multicast" not in instr, (name, instr)
     assert loads > 5
+
+
+def test_pair_kernel_waits_for_every_arrival_from_the_other_block():
+    """A commit of the pair kernel arrives in both blocks' shared memory at
+    some later time; neither block may leave before its last ones are in.  A
+    missing wait would show as a rare fault, so it is read from the source."""
+    with open(os.path.join(build_lib.PKG, "csrc", "gemm_tcgen05.cu")) as f:
+        text = f.read()
+    kernel = text[text.index("gemm_pair_tcgen05(const"):]
+    kernel = kernel[:kernel.index("tmem_dealloc_pair")]
+    assert set(re.findall(r"tc_commit_pair\(&(\w+)\[", kernel)) == {"empty", "acc_full"}
+    producer, rest = kernel.split("} else if (warp == 1) {", 1)
+    # both blocks' producers, after their last issue, take the last use of every stage
+    tail = producer[producer.rindex("tma_load_2d_pair("):]
+    waits = [line for line in tail.splitlines() if "mbar_wait_bounded(&empty[" in line]
+    assert len(waits) == 1 and "kDrainWaitNs" in waits[0]
+    before = tail[:tail.index("mbar_wait_bounded(&empty[")]
+    assert "j < n_issued" in before.splitlines()[-2] and "rank" not in before.splitlines()[-2]
+    # and both blocks' epilogues every accumulator
+    epilogue = rest[rest.index("} else {"):]
+    assert "warp_wait_uniform(&acc_full[b]" in epilogue
