@@ -492,7 +492,8 @@ snn_status_t snn_conv2d_small_dw_nhwc(int64_t M, int64_t H, int64_t W, int64_t C
  *   desc     the Leaky layer: B, N = Ho*Wo*Cout (channel-last), io_dtype
  *            SNN_BF16, save SNN_SAVE_MEM, any reset; beta_mode and thr_mode
  *            scalar or per channel with C = Cout, HW = 1
- *   X        bf16 [T*B, H, W, 1];  Wt bf16 [Cout, ldw] as above
+ *   X        bf16 [T*B, H, W, 1], at any element (2-byte alignment, as
+ *            snn_conv2d_small_fwd_nhwc takes it);  Wt bf16 [Cout, ldw] as above
  *   spk, mem bf16 [T, B, N] (out);  ckpt the spike bits, or NULL
  *   pool     bf16 [T*B, Ho/2, Wo/2, Cout] (out) and idx uint8 (out): the
  *            pooled spikes and positions, or both NULL

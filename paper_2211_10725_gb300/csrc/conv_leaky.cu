@@ -39,7 +39,8 @@
 // once per 8 steps) masks those slots in A instead.
 //
 // A block is 2 warps: its few image rows (not the whole image) are staged 8
-// steps at a time with cp.async, double-buffered, two barriers per 8 steps.
+// steps at a time with cp.async (through registers for an X that starts off a
+// 16-byte boundary), double-buffered, two barriers per 8 steps.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -74,6 +75,7 @@ struct ConvLeakyArgs {
   __nv_bfloat16* pool;  // [T*B, Ho/2, Wo/2, Cout] or null
   unsigned char* idx;   // likewise (both or neither)
   int slice;            // bytes of one step's staged rows (a multiple of 16)
+  int x_aligned;        // X starts on a 16-byte boundary (then every image does)
 };
 
 __device__ __forceinline__ void cl_cp16(uint32_t dst, const void* src) {
@@ -184,9 +186,18 @@ __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLea
     const __nv_bfloat16* src = a.X + ((int64_t)t0 * a.B + b) * img + e_lo;
     for (int v = threadIdx.x; v < n * vecs; v += kClThreads) {
       const int s = v / vecs, c = v - s * vecs;
-      if (e_lo + 8 * c < img)  // the last rows' slice may reach past the image
-        cl_cp16(sbase + (uint32_t)((buf * kClSteps + s) * a.slice + 16 * c),
-                src + (int64_t)s * a.B * img + 8 * c);
+      if (e_lo + 8 * c >= img) continue;  // the last rows' slice may reach past the image
+      const uint32_t at = (uint32_t)((buf * kClSteps + s) * a.slice + 16 * c);
+      const __nv_bfloat16* x = src + (int64_t)s * a.B * img + 8 * c;
+      if (a.x_aligned) {
+        cl_cp16(sbase + at, x);
+      } else {  // a view off the 16-byte boundary: element by element, through registers
+        const unsigned short* e = reinterpret_cast<const unsigned short*>(x);
+        uint32_t w[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) w[k] = (uint32_t)e[2 * k] | ((uint32_t)e[2 * k + 1] << 16);
+        *reinterpret_cast<uint4*>(sm + at) = make_uint4(w[0], w[1], w[2], w[3]);
+      }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
@@ -371,7 +382,7 @@ extern "C" snn_status_t snn_conv2d_small_leaky_fwd_nhwc(
   ConvLeakyArgs a{};
   if (!mode(d->beta_mode, &a.beta_ch) || !mode(d->thr_mode, &a.thr_ch)) return SNN_ERR_UNSUPPORTED;
   if (!X || !Wt || !beta || !thr || !spk || !mem) return SNN_ERR_INVALID_ARG;
-  if (!cl_al16(X) || !cl_al16(spk) || !cl_al16(mem) || (ckpt && !cl_al16(ckpt)) ||
+  if ((reinterpret_cast<uintptr_t>(X) & 1u) || !cl_al16(spk) || !cl_al16(mem) || (ckpt && !cl_al16(ckpt)) ||
       (pool && (!cl_al16(pool) || !cl_al16(idx))) || (reinterpret_cast<uintptr_t>(Wt) & 1u))
     return SNN_ERR_ALIGNMENT;
   a.T = (int)d->T;
@@ -392,6 +403,7 @@ extern "C" snn_status_t snn_conv2d_small_leaky_fwd_nhwc(
   a.bits_row = ((d->B * d->N + 7) / 8 + 15) / 16 * 16;
   a.pool = static_cast<__nv_bfloat16*>(pool);
   a.idx = idx;
+  a.x_aligned = cl_al16(X);
   const int64_t Wp = Wo / 2, Pp = (Ho / 2) * Wp;
   const int64_t parts = (Pp + 8 * kClWarps - 1) / (8 * kClWarps);
   // image rows a block can touch: its consecutive windows span at most

@@ -8,6 +8,7 @@ import torch
 
 from paper_2211_10725_gb300 import snn
 from paper_2211_10725_gb300 import workloads as W
+from paper_2211_10725_gb300.csnn import ConvSNN
 
 pytestmark = pytest.mark.gpu
 
@@ -154,3 +155,32 @@ def test_patch_rows_and_their_gradient_over_shapes(M, H, Wd, C, k, Kpad, cuda_de
     for t in range(k * k):
         s[:, t // k: t // k + Ho, t % k: t % k + Wo] += d[..., t * C:(t + 1) * C].float()
     assert torch.equal(dX.cpu(), s.to(torch.bfloat16))
+
+
+@pytest.mark.parametrize("offset", [1, 4])   # 2 and 8 bytes off a 16-byte boundary
+def test_network_takes_an_input_view_at_any_element(offset, cuda_device):
+    """A fused network steps on a view into a larger buffer, wherever it
+    starts: the same spikes, trace and pooling as on a copy of its own."""
+    w = W.CSNN_C4.scaled(T=9, B=2)
+    inp = W.make_conv_inputs(w)
+    X = inp["X"].to(cuda_device).reshape(w.T * w.B, w.H, w.W, w.Cin).contiguous()
+    buf = torch.zeros(X.numel() + 8, dtype=X.dtype, device=cuda_device)
+    view = buf[offset:offset + X.numel()].view(X.shape)
+    view.copy_(X)
+    labels = inp["labels"].to(cuda_device)
+    nets = []
+    for x in (X, view):
+        net = ConvSNN(w, inp["convs"], inp["Wfc"], device=cuda_device, save="fused")
+        assert net.direct_scan[0]
+        net.step(x, labels)
+        nets.append(net)
+    torch.cuda.synchronize()
+    a, b = nets
+    assert int(a.layers[0].spk.float().sum()) > 0
+    for got, ref in ((b.layers[0].spk, a.layers[0].spk), (b.layers[0].mem, a.layers[0].mem),
+                     (b.pool[0], a.pool[0]), (b.idx[0], a.idx[0]), (b.loss, a.loss)):
+        assert torch.equal(got, ref)
+    # the weight gradient of such a view is another kernel's: both are fp32
+    # sums of the same products
+    err = (b.dW[0].double() - a.dW[0].double()).norm()
+    assert float(err) <= 1e-5 * float(a.dW[0].double().norm())
