@@ -210,9 +210,10 @@ snn_status_t snn_leaky_fwd(const snn_scan_desc* desc, const void* I, const float
  * where d u_{t+1}/d u_t = beta (subtract/none) or beta*(1-z_t) (zero) and
  * d u_{t+1}/d z_t = -thr (subtract), -beta*u_t (zero), 0 (none).
  * Parameter sums are accumulated in fp32 per lane and reduced across lanes
- * in a fixed order (deterministic): tens of lanes in fp32, everything above
- * them in compensated fp32 (a sum and the rounding error of its additions,
- * two-sum).
+ * in a fixed order (deterministic): at most five plain additions deep within
+ * a warp of the scan, or a sample split's (B+7)/8 per-neuron lanes, everything
+ * above them in compensated fp32 (a sum and the rounding error of its
+ * additions, two-sum).
  * SNN_SAVE_RECOMPUTE replays Eq. (4) from each checkpoint bit for bit as the
  * forward evaluated it.  With ckpt_every 8 (any dtype pair), 12 or 16 (bf16
  * or fp16 input and io), no grad_mem, a reset other than SNN_RESET_NONE and B*N

@@ -3,14 +3,13 @@
 // per warp and channel, or per run of a channel's lanes, see PART_* in
 // scan_kernels.cuh) into the parameter's shape:
 // scalar, per neuron [N] (sum over b) or per channel [C] (sum over b and the
-// channel's H*W positions).  Each thread adds its own run of lanes in fp32
-// (tens of terms: an error of a few 1e-6 of their magnitudes), and
-// everything above that in compensated fp32: a running sum and the rounding
-// error of its additions (Knuth's two-sum), close to fp64's accuracy for
-// these sums without fp64 arithmetic, which is slow on this part (with one
-// fp64 add per lane the per-neuron reduction of the 524,288-lane workload
-// took 11.5 us).  Every sum is taken in a fixed order, so repeated calls
-// give identical bits.
+// channel's H*W positions).  The sums are taken in compensated fp32: a running
+// sum and the rounding error of its additions (Knuth's two-sum), close to
+// fp64's accuracy for these sums without fp64 arithmetic, which is slow on
+// this part (with one fp64 add per lane the per-neuron reduction of the
+// 524,288-lane workload took 11.5 us); only the per-neuron reduction adds each
+// split's samples in plain fp32 first.  Every sum is taken in a fixed order,
+// so repeated calls give identical bits.
 //
 // One launch reduces every parameter that shares a layout (blockIdx.z picks
 // the parameter).  Scalar and per-channel: block (x, y) of a parameter sums
@@ -29,7 +28,7 @@ namespace snn {
 namespace {
 
 constexpr int kRedThreads = 256;
-constexpr int64_t kChanChunk = 8192;  // lanes per block of the channel-last reduction (32 per thread)
+constexpr int64_t kChanChunk = 8192;  // partials per block of the channel-last reduction (32 per thread)
 constexpr int64_t kNeuronSplit = 8;
 
 // The lanes' values added in a fixed tree, in every lane.
@@ -83,12 +82,12 @@ __global__ void __launch_bounds__(kRedThreads) reduce_scalar(ReduceJobs js, int6
   const int S = gridDim.y;
   const int64_t lo = (int64_t)blockIdx.y * chunk;
   const int64_t hi = min(L, lo + chunk);
-  // a thread's run of lanes (16 at the default chunk) in fp32, in order;
-  // everything above compensated
-  float acc = 0.0f;
+  // a thread's run (16 partials at the default chunk, each of them a whole
+  // warp's lanes behind a staged scan) in order
+  float2 acc = make_float2(0.0f, 0.0f);
 #pragma unroll 8
-  for (int64_t l = lo + threadIdx.x; l < hi; l += kRedThreads) acc += j.part[l];
-  const float2 s = block_sum(make_float2(acc, 0.0f), sh);
+  for (int64_t l = lo + threadIdx.x; l < hi; l += kRedThreads) acc = two_add(acc, j.part[l]);
+  const float2 s = block_sum(acc, sh);
   if (S == 1) {  // the group's only block
     if (threadIdx.x == 0) j.out[0] = pair_value(s);
     return;
@@ -145,7 +144,7 @@ __global__ void __launch_bounds__(kRedThreads) reduce_per_channel(ReduceJobs js,
   const int64_t c = blockIdx.x, s = blockIdx.y, S = gridDim.y;
   const int64_t R = N / (C * HW);
   const int64_t runs = (B * R - s + S - 1) / S;  // runs j = s + q*S, q < runs
-  float acc = 0.0f;  // a thread's elements in fp32, in order; the block's compensated
+  float2 acc = make_float2(0.0f, 0.0f);  // a thread's elements, in order
   if (runs * HW <= INT_MAX / 2 && B * R <= INT_MAX / 2) {  // the same in 32-bit divisions
     const int n = (int)(runs * HW), hw = (int)HW, rr = (int)R;
 #pragma unroll 4
@@ -153,17 +152,17 @@ __global__ void __launch_bounds__(kRedThreads) reduce_per_channel(ReduceJobs js,
       const int q = e / hw, h = e - q * hw;
       const int jr = (int)s + q * (int)S;
       const int b = jr / rr, r = jr - b * rr;
-      acc += j.part[b * N + (r * C + c) * HW + h];
+      acc = two_add(acc, j.part[b * N + (r * C + c) * HW + h]);
     }
   } else {
     for (int64_t e = threadIdx.x; e < runs * HW; e += blockDim.x) {
       const int64_t q = e / HW, h = e - q * HW;
       const int64_t jr = s + q * S;
       const int64_t b = jr / R, r = jr - b * R;
-      acc += j.part[b * N + (r * C + c) * HW + h];
+      acc = two_add(acc, j.part[b * N + (r * C + c) * HW + h]);
     }
   }
-  const float2 v = block_sum(make_float2(acc, 0.0f), sh);
+  const float2 v = block_sum(acc, sh);
   if (S == 1) {
     if (threadIdx.x == 0) j.out[c] = pair_value(v);
     return;
@@ -200,12 +199,11 @@ __global__ void __launch_bounds__(kRedThreads) reduce_channel_last(ReduceJobs js
   const ReduceJob& j = js.job[blockIdx.z];
   const int64_t lo = (int64_t)blockIdx.x * chunk;
   const int64_t hi = min(L, lo + chunk);
-  // a thread's run of lanes (32 at kChanChunk) in fp32, everything above
-  // compensated
-  float acc = 0.0f;
+  // a thread's run (32 partials at kChanChunk), in order
+  float2 acc = make_float2(0.0f, 0.0f);
 #pragma unroll 8
-  for (int64_t l = lo + threadIdx.x; l < hi; l += kRedThreads) acc += j.part[l];
-  sh[threadIdx.x] = make_float2(acc, 0.0f);
+  for (int64_t l = lo + threadIdx.x; l < hi; l += kRedThreads) acc = two_add(acc, j.part[l]);
+  sh[threadIdx.x] = acc;
   __syncthreads();
   if ((int)threadIdx.x < C) {
     float2 t = make_float2(0.0f, 0.0f);

@@ -572,8 +572,10 @@ __device__ __forceinline__ void initial_state(const ScanArgs& a, int64_t l, cons
 
 // One parameter's gradient partials of a consumer warp, in the layout the
 // launch chose; every lane of the warp calls it (an inactive thread adds
-// zeros).  gw: the warp's index among the launch's consumer warps.  Tens of
-// terms are added in fp32, more in compensated fp32.
+// zeros).  gw: the warp's index among the launch's consumer warps.  Plain
+// fp32 where a sum is at most five additions deep (a thread's own lanes; the
+// channels of a warp), compensated above that; the reduction that follows is
+// compensated throughout.
 template <int V>
 __device__ __forceinline__ void store_partials(const ScanArgs& a, float* part, int kind, float (&v)[V],
                                                int64_t l, bool active, int64_t gw, int lid) {
@@ -584,7 +586,7 @@ __device__ __forceinline__ void store_partials(const ScanArgs& a, float* part, i
 #pragma unroll
   for (int k = 0; k < V; ++k)
     if (!active) v[k] = 0.0f;
-  if (kind == PART_CHANNELS) {  // threads C / V apart hold the same channels: at most 16 terms
+  if (kind == PART_CHANNELS) {  // threads C / V apart hold the same channels: a tree of at most 32 terms
     const int period = (int)a.C / V;
     for (int d = period; d < 32; d <<= 1)
 #pragma unroll
@@ -602,9 +604,10 @@ __device__ __forceinline__ void store_partials(const ScanArgs& a, float* part, i
     if (lid == 0) part[gw] = pair_value(p);
     return;
   }
-  const int group = a.part_q / V;  // threads that add up: at most 32 terms
-  for (int d = 1; d < group; d <<= 1) s += __shfl_xor_sync(0xffffffffu, s, d);
-  if (active && (lid & (group - 1)) == 0) part[l / a.part_q] = s;
+  const int group = a.part_q / V;  // threads that add up: at most 8
+  float2 p = make_float2(s, 0.0f);
+  for (int d = 1; d < group; d <<= 1) p = pair_add(p, shfl_xor_pair(p, d));
+  if (active && (lid & (group - 1)) == 0) part[l / a.part_q] = pair_value(p);
 }
 
 // ---------------------------------------------------------------------------

@@ -161,7 +161,7 @@ def test_patch_rows_and_their_gradient_over_shapes(M, H, Wd, C, k, Kpad, cuda_de
 def test_network_takes_an_input_view_at_any_element(offset, cuda_device):
     """A fused network steps on a view into a larger buffer, wherever it
     starts: the same spikes, trace and pooling as on a copy of its own."""
-    w = W.CSNN_C4.scaled(T=9, B=2)
+    w = W.CSNN_C4.scaled(T=9, B=8)
     inp = W.make_conv_inputs(w)
     X = inp["X"].to(cuda_device).reshape(w.T * w.B, w.H, w.W, w.Cin).contiguous()
     buf = torch.zeros(X.numel() + 8, dtype=X.dtype, device=cuda_device)
