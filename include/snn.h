@@ -285,6 +285,12 @@ snn_status_t snn_dense_layer_fwd(int64_t M, int64_t K, int64_t N, const void* X,
  * the partials are added in a fixed order (the same bits on every call). */
 size_t snn_dense_workspace_bytes(int64_t M, int64_t K, int64_t N);
 
+/* The columns (128, 192 or 256) of the two-CTA tiles that a product of the
+ * dense layer runs on, on a GPU of `sms` SMs, or 0 where single CTAs are
+ * faster: product 0 the forward, 1 dX, 2 dW.  -1 for invalid arguments.  Host
+ * only (the choice for 16-byte aligned buffers), for tests and planning. */
+int snn_dense_pair_width(int64_t M, int64_t K, int64_t N, int product, int sms);
+
 /*
  * Backward of snn_dense_layer_fwd, given dI = dL/dI (bf16 [M, N], e.g. the
  * grad_I of a scan with bf16 io):

@@ -603,36 +603,37 @@ cudaError_t launch_pair(const CUtensorMap& ta, const CUtensorMap& tb, const CUte
                             dim3(kThreads), pair_smem_bytes<BN>(), st, ta, tb, td, g);
 }
 
-// D[M, N] = A[M, K] * B[N, K]^T.  A is stored [M, K] row-major (K-major) or,
-// with A_MN, [K, M] row-major; B likewise [N, K] or, with B_MN, [K, N].
-// N tile: the widest the output needs (64, 128 or 192 for an MN-major B),
-// and 64 rather than 128 when 128-wide tiles would leave most SMs idle.
-template <bool OUT_BF16, bool A_MN = false, bool B_MN = false>
-cudaError_t gemm_tn(const void* A, const void* B, void* D, int M, int N, int K, int* status,
-                    cudaStream_t st, int ksplit = 1, int bn_force = 0) {
+// N tile on single CTAs: the widest the output needs (64, 128 or 192 for an
+// MN-major B), and 64 rather than 128 when 128-wide tiles would leave most
+// SMs idle.  force: a width the caller chose, or 0.
+template <bool B_MN>
+int single_width(int M, int N, int K, int force, int sms) {
+  if (force > 0) return force;
+  if (N <= 16 && !B_MN) return 16;
+  if (N <= 32 && !B_MN) return 32;
+  if (N <= 64) return 64;
+  // an MN-major B wider than two 128-column tiles: 192-wide tiles when
+  // they need fewer tiles (each re-reads its A rows once)
+  if (B_MN && N > 256 && (N + 191) / 192 < (N + 127) / 128) return 192;
+  const int64_t tiles128 = (int64_t)((N + 127) / 128) * ((M + BM - 1) / BM);
+  if (tiles128 < (int64_t)sms * kCtasPerSm) return 64;
   // a 128 x 256 tile keeps the tensor core busier per instruction (about
   // 1.6x the rate of 128 x 128 at large K); below K = 512 the per-tile
   // fixed costs dominate and the narrower tile's parallelism wins
-  int bn = (!B_MN && N > 128 && K >= 512) ? 256 : 128;
-  if (bn_force > 0) bn = bn_force;
-  else if (N <= 16 && !B_MN) bn = 16;
-  else if (N <= 32 && !B_MN) bn = 32;
-  else if (N <= 64) bn = 64;
-  // an MN-major B wider than two 128-column tiles: 192-wide tiles when
-  // they need fewer tiles (each re-reads its A rows once)
-  else if (B_MN && N > 256 && (N + 191) / 192 < (N + 127) / 128) bn = 192;
-  else {
-    int dev = 0, sms = 152;
-    if (cudaGetDevice(&dev) == cudaSuccess)
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t tiles128 = (int64_t)((N + 127) / 128) * ((M + BM - 1) / BM);
-    if (tiles128 < (int64_t)sms * kCtasPerSm) bn = 64;
-  }
+  return (!B_MN && N > 128 && K >= 512) ? 256 : 128;
+}
+
+// D[M, N] = A[M, K] * B[N, K]^T.  A is stored [M, K] row-major (K-major) or,
+// with A_MN, [K, M] row-major; B likewise [N, K] or, with B_MN, [K, N].
+template <bool OUT_BF16, bool A_MN = false, bool B_MN = false>
+cudaError_t gemm_tn(const void* A, const void* B, void* D, int M, int N, int K, int* status,
+                    cudaStream_t st, int ksplit = 1, int bn_force = 0) {
+  DeviceInfo info;
+  const bool known = device_info(&info) == cudaSuccess;
+  const int bn = single_width<B_MN>(M, N, K, bn_force, known ? info.sms : 152);
   CUtensorMap ta, tb;
   const bool okA = A_MN ? make_map(&ta, A, K, M, 64) : make_map(&ta, A, M, K, BM);
-  DeviceInfo info;
-  if (device_info(&info) == cudaSuccess && ((int64_t)N * (OUT_BF16 ? 2 : 4)) % 16 == 0 &&
-      (reinterpret_cast<uintptr_t>(D) & 15u) == 0) {
+  if (known && ((int64_t)N * (OUT_BF16 ? 2 : 4)) % 16 == 0 && (reinterpret_cast<uintptr_t>(D) & 15u) == 0) {
     const int w = pair_width<OUT_BF16, B_MN>(M, N, K, ksplit, bn, info.sms);
     CUtensorMap td;
     if (w > 0 && okA && (B_MN ? make_map(&tb, B, K, N, 64) : make_map(&tb, B, N, K, w / 2)) &&
@@ -773,6 +774,17 @@ size_t snn_dense_workspace_bytes(int64_t M, int64_t K, int64_t N) {
   // split-K partials of dW when the weight gradient is split
   const int S = dw_splits(M, K, N);
   return 256 + (S > 1 ? round256((size_t)S * N * K * sizeof(float)) : 0);
+}
+
+int snn_dense_pair_width(int64_t M, int64_t K, int64_t N, int product, int sms) {
+  if (check_dims(M, K, N) != SNN_OK || product < 0 || product > 2 || sms < 1) return -1;
+  if (M == 0 || K == 0 || N == 0) return 0;
+  const int m = (int)M, k = (int)K, n = (int)N;
+  if (product == 0)
+    return n % 4 != 0 ? 0 : pair_width<false, false>(m, n, k, 1, single_width<false>(m, n, k, 0, sms), sms);
+  if (product == 1) return pair_width<true, true>(m, k, n, 1, single_width<true>(m, k, n, 0, sms), sms);
+  const DwPlan plan = dw_plan(M, K, N);
+  return pair_width<false, true>(n, k, m, plan.S, single_width<true>(n, k, m, plan.bn, sms), sms);
 }
 
 snn_status_t snn_dense_layer_fwd(int64_t M, int64_t K, int64_t N, const void* X, const void* W,

@@ -75,6 +75,7 @@ _SIGS = {
     "snn_rleaky_bwd": ([ctypes.POINTER(ScanDesc)] + [_P] * 17 + [ctypes.c_size_t, _P], ctypes.c_int),
     "snn_dense_layer_fwd": ([ctypes.c_int64] * 3 + [_P] * 4 + [ctypes.c_size_t, _P], ctypes.c_int),
     "snn_dense_workspace_bytes": ([ctypes.c_int64] * 3, ctypes.c_size_t),
+    "snn_dense_pair_width": ([ctypes.c_int64] * 3 + [ctypes.c_int] * 2, ctypes.c_int),
     "snn_dense_layer_bwd": ([ctypes.c_int64] * 3 + [_P] * 6 + [ctypes.c_size_t, _P], ctypes.c_int),
     "snn_rate_ce_workspace_bytes": ([ctypes.c_int64], ctypes.c_size_t),
     "snn_kernel_launches": ([], ctypes.c_uint64),
@@ -267,6 +268,12 @@ def snn_leaky_bwd_noalloc(desc, I, ckpt, mem, spk, beta, thr, mem0, grad_spk, gr
 
 def snn_dense_workspace_bytes(M: int, K: int, N: int) -> int:
     return load_library().snn_dense_workspace_bytes(M, K, N)
+
+
+def snn_dense_pair_width(M: int, K: int, N: int, product: int, sms: int) -> int:
+    """Columns of the two-CTA tiles a product of the dense layer (0 forward, 1
+    dX, 2 dW) runs on with `sms` SMs; 0: single CTAs."""
+    return load_library().snn_dense_pair_width(M, K, N, product, sms)
 
 
 def snn_dense_layer_fwd(X, W, I, ws, stream=None):
