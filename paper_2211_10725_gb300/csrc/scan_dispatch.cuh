@@ -23,6 +23,12 @@ inline bool few_lanes(int64_t L) {
   return device_info(&d) == cudaSuccess && L < 2048 * (int64_t)d.sms;
 }
 
+// Lanes of the plain kernels from which other warps hide a load (see there).
+inline bool many_lanes(int64_t L) {
+  DeviceInfo d;
+  return device_info(&d) == cudaSuccess && L >= kPlainManyLanes * (int64_t)d.sms;
+}
+
 template <bool SYN, typename TI, typename TO, int RESET, bool REC, int VL, bool STRIPS, bool CK>
 cudaError_t fwd_staged_ck(ScanArgs a, cudaStream_t st, bool* launched) {
   const void* k = (const void*)scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, STRIPS, CK>;
@@ -130,14 +136,22 @@ cudaError_t bwd_staged(ScanArgs a, cudaStream_t st, bool* launched) {
   return bwd_staged_vl<SYN, RECOMP, TI, TO, RESET, SG, KC, REC, kLanes<SYN>>(a, st, launched);
 }
 
-template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int REC>
-cudaError_t bwd_plain(ScanArgs a, cudaStream_t st) {
+template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int REC, int AHEAD>
+cudaError_t bwd_plain_ahead(ScanArgs a, cudaStream_t st) {
   const int threads = 128;
   const size_t smem = RECOMP ? (size_t)a.K * threads * 4 * (SYN ? 2 : 1) : 0;
-  const cudaError_t e = ensure_smem((const void*)scan_bwd_plain<SYN, RECOMP, TI, TO, RESET, SG, REC>, smem);
+  const auto kernel = scan_bwd_plain<SYN, RECOMP, TI, TO, RESET, SG, REC, AHEAD>;
+  const cudaError_t e = ensure_smem((const void*)kernel, smem);
   if (e != cudaSuccess) return e;
-  return launch_pdl(scan_bwd_plain<SYN, RECOMP, TI, TO, RESET, SG, REC>,
-                    dim3((unsigned)ceil_div(a.L, threads)), dim3(threads), smem, st, a);
+  return launch_pdl(kernel, dim3((unsigned)ceil_div(a.L, threads)), dim3(threads), smem, st, a);
+}
+
+template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int REC>
+cudaError_t bwd_plain(ScanArgs a, cudaStream_t st) {
+  constexpr int few = RECOMP ? kPlainAheadSeg : kPlainAhead;
+  constexpr int many = RECOMP ? kPlainAheadSegMany : kPlainAheadMany;
+  return many_lanes(a.L) ? bwd_plain_ahead<SYN, RECOMP, TI, TO, RESET, SG, REC, many>(a, st)
+                         : bwd_plain_ahead<SYN, RECOMP, TI, TO, RESET, SG, REC, few>(a, st);
 }
 
 template <bool SYN, bool RECOMP, typename TI, typename TO>

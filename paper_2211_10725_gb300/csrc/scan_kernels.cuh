@@ -1306,34 +1306,61 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_bwd_staged(const ScanA
 // ---------------------------------------------------------------------------
 // Plain kernels: one lane per thread, direct loads, any shape.
 // The recurrence needs the rows one after another, but their loads depend on
-// nothing, so each thread keeps 16 to 32 steps' loads in flight (8 to 16 in
-// a checkpoint segment): with one step's load on the chain at a time a step cost a memory
-// latency.  T = 75, 33 x 1001 lanes in half precision, both passes: 52 us;
-// with 8 to 16 steps' loads ahead 33, with the modes compiled in and pointers
-// that walk instead of 64-bit address products 25.2, and with 16 to 32 steps
-// 24.5 (4 us at 6.7 TB/s: the lanes are one or two warps a scheduler, so a
-// step's instructions bound it).  Segments of 12 steps took 44.6 us with 16
-// ahead, 37.5 with 8.
+// nothing, so a thread of a small layer keeps 8 to 16 steps' loads in flight
+// (4 to 8 in a checkpoint segment): with one step's load on the chain at a
+// time a step cost a memory latency.  T = 75, 33 x 1001 lanes in half
+// precision, both passes: 52 us; with loads ahead 33, with the modes compiled
+// in and pointers that walk instead of 64-bit address products 25.2, and
+// whole blocks without a test per step 20.9 (4 us at 6.7 TB/s: the lanes are
+// one or two warps a scheduler, so a step's instructions bound it).
+//
+// From two warps a scheduler the other warps hide a load and the look-ahead's
+// registers cost them: the store-mode backward keeps 4 to 8 steps in flight
+// there, and the recompute backward (32 registers instead of 56) none.
+// us, T = 75, rows of 1001 lanes:
+//   samples                                33     101     331    1503
+//   bf16 recompute, backward, one step   28.4    31.4   127.9   374.6
+//                             4 ahead    22.6    38.8   113.3   451.5
+//   fp32 Synaptic, both passes, 16       41.8    97.7   334.6  1467.7
+//                               4 ahead  44.2    70.0   241.1   959.3
+// One step at a time is slower by an eighth at 331 samples, where the layer
+// just fills the GPU once, and faster by a fifth beyond.
 // ---------------------------------------------------------------------------
 
-constexpr int kPlainAhead = 16;    // whole sequences
-constexpr int kPlainAheadSeg = 8;  // checkpoint segments, most of them shorter than 16 steps
+constexpr int kPlainAhead = 8;         // forward, store-mode backward
+constexpr int kPlainAheadMany = 4;     // store-mode backward of many lanes
+constexpr int kPlainAheadSeg = 4;      // checkpoint segments
+constexpr int kPlainAheadSegMany = 1;  // of many lanes
+constexpr int kPlainManyLanes = 256;   // lanes per SM: two warps a scheduler
 
 // step(i, item) for i = 0 .. n-1 in order, item = load(i) issued A to 2*A
-// steps before it is used.
+// steps before it is used, or (A = 1) right before.  Whole blocks run without a
+// test per step.
 template <typename Item, int A, typename Load, typename Step>
 __device__ __forceinline__ void plain_steps(int64_t n, Load load, Step step) {
+  if constexpr (A == 1) {
+    for (int64_t i = 0; i < n; ++i) step(i, load(i));
+    return;
+  }
   Item cur[A], next[A];
 #pragma unroll
   for (int k = 0; k < A; ++k)
     if (k < n) cur[k] = load(k);
   for (int64_t i = 0; i < n; i += A) {
+    if (n - i >= 2 * A) {
 #pragma unroll
-    for (int k = 0; k < A; ++k)
-      if (i + A + k < n) next[k] = load(i + A + k);
+      for (int k = 0; k < A; ++k) next[k] = load(i + A + k);
 #pragma unroll
-    for (int k = 0; k < A; ++k)
-      if (i + k < n) step(i + k, cur[k]);
+      for (int k = 0; k < A; ++k) step(i + k, cur[k]);
+    } else {
+      const int left = (int)(n - i);
+#pragma unroll
+      for (int k = 0; k < A; ++k)
+        if (A + k < left) next[k] = load(i + A + k);
+#pragma unroll
+      for (int k = 0; k < A; ++k)
+        if (k < left) step(i + k, cur[k]);
+    }
 #pragma unroll
     for (int k = 0; k < A; ++k) cur[k] = next[k];
   }
@@ -1390,7 +1417,7 @@ __global__ void __launch_bounds__(128) scan_fwd_plain(const ScanArgs a) {
   if (SYN && a.syn_final) a.syn_final[l] = i;
 }
 
-template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int REC>
+template <bool SYN, bool RECOMP, typename TI, typename TO, int RESET, int SG, int REC, int AHEAD>
 __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
   extern __shared__ __align__(16) float segbuf[];  // [K][blockDim] u, then i
   grid_dep_wait();
@@ -1421,7 +1448,7 @@ __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
     struct Item {
       TO g, u, z, i, m;
     };
-    plain_steps<Item, kPlainAhead>(
+    plain_steps<Item, AHEAD>(
         a.T,
         [&](int64_t) {
           Item it;
@@ -1466,14 +1493,14 @@ __global__ void __launch_bounds__(128) scan_bwd_plain(const ScanArgs a) {
         i = s0;
         z = have_mem0 && (m0 > thr);
       }
-      plain_steps<TI, kPlainAheadSeg>(
+      plain_steps<TI, AHEAD>(
           t1 - t0, [&](int64_t j) { return I[(t0 + j) * a.L]; },
           [&](int64_t j, const TI& x) {
             fwd_step<SYN, RESET, REC>(a.reset, beta, thr, alpha, Elem<TI>::load1(&x), u, z, i, a.rec != 0);
             su[j * blockDim.x] = u;
             if (SYN) si[j * blockDim.x] = i;
           });
-      plain_steps<Item, kPlainAheadSeg>(
+      plain_steps<Item, AHEAD>(
           t1 - t0,
           [&](int64_t j) {
             const int64_t off = (t1 - 1 - j) * a.L;
