@@ -493,9 +493,11 @@ snn_status_t snn_conv2d_small_dw_nhwc(int64_t M, int64_t H, int64_t W, int64_t C
  * First-layer convolution with its Leaky scan and 2x2 max pooling in one
  * kernel (the CSNN's 5x5 filters over the 1-channel input map; Eqs. 3-4):
  * the same results as snn_conv2d_small_fwd_nhwc, snn_leaky_fwd and
- * snn_maxpool2_fwd_nhwc in turn wherever the currents' sums are exact in
- * fp32 (spikes times bf16 filters), else within fp32 rounding of the
- * currents; the currents are never written.
+ * snn_maxpool2_fwd_nhwc in turn for 3x3 filters, and for 5x5 filters wherever
+ * the currents' sums are exact in fp32 (spikes times bf16 filters); else a
+ * 5x5 current is within 25 roundings (2^-24 of its summed magnitudes each),
+ * and on average closer than the separate convolution's multiply-adds.  The
+ * currents are never written.
  *   desc     the Leaky layer: B, N = Ho*Wo*Cout (channel-last), io_dtype
  *            SNN_BF16, save SNN_SAVE_MEM, any reset; beta_mode and thr_mode
  *            scalar or per channel with C = Cout, HW = 1

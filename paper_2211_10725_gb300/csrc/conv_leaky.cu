@@ -23,6 +23,15 @@
 // thread.  A first version with one pixel per row had to load two words and
 // permute them for every odd pixel, and issued 270 instructions per 16
 // pixels a step (46 us); this one 320 per 32.
+// The tensor core truncates its sums, so a patch's two products start from
+// zero and are added in rounded fp32.  Error of a current over its summed
+// magnitudes, rms in units of 2^-24, uniform pixels: 0.119 so, 0.145 with the
+// first sum handed to the second product, 0.136 with fp32 multiply-adds
+// (normal pixels 0.129, 0.149, 0.132); 30.2 us at T = 25, B = 128.
+// The 9 taps of a 3x3 filter are fp32 multiply-adds in filter order, the
+// separate convolution's bits: as one product their error was 0.076 against
+// 0.066, and a product for each filter row with compensated sums between them
+// took 59 us where this takes 38.9 (three kernels 88).
 // A tcgen05 tile (M = 128, 64-deep swizzled K blocks) would need the patch
 // rows built in shared memory, which is the traffic this avoids; the product
 // is 8 mma per 32 pixels and not what bounds the kernel.
@@ -48,7 +57,7 @@
 #include <cstdint>
 #include <type_traits>
 
-#include "launch.cuh"
+#include "scan_host.cuh"
 #include "scan_kernels.cuh"
 #include "snn.h"
 
@@ -82,14 +91,15 @@ __device__ __forceinline__ void cl_cp16(uint32_t dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2],
-                                         float c0, float c1, float c2, float c3) {
+// A product from zero: a tensor core truncates its sums, so the two k-steps
+// of a patch are added in rounded fp32 instead of the first being handed to
+// the second.
+__device__ __forceinline__ void mma_bf16_zero(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-      "{%8, %9}, {%10, %11, %12, %13};"
+      "{%8, %9}, {%10, %10, %10, %10};"
       : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(c0), "f"(c1), "f"(c2),
-        "f"(c3));
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]), "f"(0.0f));
 }
 
 // fwd_pair with the reset-to-zero state kept as (1 - z)*u (exact: u or a
@@ -115,7 +125,8 @@ template <int KS, int RESET>
 __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLeakyArgs a) {
   constexpr int PR = (KS + 1) / 2;          // words per filter row
   constexpr int PAIRS = KS * PR;            // words per patch: 15 (5x5), 6 (3x3)
-  constexpr int KSTEPS = (PAIRS + 7) / 8;   // k16 steps: 2, 1
+  constexpr bool MMA = KS == 5;
+  constexpr int KSTEPS = MMA ? (PAIRS + 7) / 8 : 0;  // k16 steps
   extern __shared__ __align__(16) unsigned char sm[];
   const int lid = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lid >> 2, q = lid & 3;
@@ -136,7 +147,7 @@ __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLea
   // B fragments.  Column 8*nb + c belongs to thread c / 2 of the quad, as its
   // value v = 2*nb + (c & 1): pixel (c / 2) & 1 of the pair, channel 8*(c /
   // 4) + v
-  uint32_t wb[KSTEPS][4][2];
+  uint32_t wb[MMA ? KSTEPS : 1][4][2];
   {
     const int ch8 = 8 * (g >> 2), right = (g >> 1) & 1;
     const unsigned short* w = reinterpret_cast<const unsigned short*>(a.Wt);
@@ -157,7 +168,7 @@ __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLea
         }
   }
   // byte offset of the thread's A words from the pair's first pixel
-  uint32_t aoff[KSTEPS][2];
+  uint32_t aoff[MMA ? KSTEPS : 1][2];
 #pragma unroll
   for (int ks = 0; ks < KSTEPS; ++ks)
 #pragma unroll
@@ -165,6 +176,13 @@ __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLea
       const int pi = ks * 8 + q + 4 * h, ky = pi / PR, s = 2 * (pi % PR);
       aoff[ks][h] = pi < PAIRS ? 2u * (uint32_t)(ky * a.W + s) : 0u;
     }
+  // 3x3: the filters as fp32 [tap][channel] behind the staged rows
+  const uint32_t w_addr = smem_u32(sm) + (uint32_t)(2 * kClSteps * a.slice);
+  if constexpr (!MMA) {
+    float* wsm = reinterpret_cast<float*>(sm + 2 * kClSteps * a.slice);
+    for (int e = threadIdx.x; e < KS * KS * kClCout; e += kClThreads)
+      wsm[e] = __bfloat162float(a.Wt[(int64_t)(e % kClCout) * a.ldw + e / kClCout]);
+  }
   const int right = q & 1, ch0 = 8 * (q >> 1);  // this thread's pixel of the pair, first channel
   float2 beta[4], negthr[4];
 #pragma unroll
@@ -216,48 +234,78 @@ __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLea
   // one time step from the staged rows at p0; MASK: slots outside the
   // pixel's window are cleared from A (else they only meet zeros in B)
   auto step = [&](uint32_t p0, auto mask) {
-    constexpr bool MASK = decltype(mask)::value;
-    float c[4][4];
+    float2 cur[2][4];  // currents of the upper and lower pixel, 4 pairs of channels
+    if constexpr (!MMA) {
+      float x[KS + 1][KS];  // this pixel's windows of both rows
 #pragma unroll
-    for (int ks = 0; ks < KSTEPS; ++ks) {
-      uint32_t av[4];
+      for (int y = 0; y <= KS; ++y) {
+        uint32_t w0, w1;
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w0) : "r"(p0 + y * row_b));
+        asm volatile("ld.shared.u32 %0, [%1];" : "=r"(w1) : "r"(p0 + y * row_b + 4));
+        const uint32_t w = __funnelshift_r(w0, w1, 16 * right);
+        x[y][0] = __uint_as_float(w << 16);
+        x[y][1] = __uint_as_float(w & 0xffff0000u);
+        x[y][2] = __uint_as_float(right ? w1 & 0xffff0000u : w1 << 16);
+      }
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
+      for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int r = 0; r < 2; ++r)  // a0: (upper row, h 0), a1: (lower, 0), a2: (upper, 1), ...
-          asm volatile("ld.shared.u32 %0, [%1];" : "=r"(av[2 * h + r]) : "r"(p0 + aoff[ks][h] + r * row_b));
-      if (!MASK) {
+        for (int j = 0; j < 4; ++j) cur[r][j] = f2(0.0f);
 #pragma unroll
-        for (int nb = 0; nb < 4; ++nb) {
-          if (ks == 0) mma_bf16(c[nb], av, wb[ks][nb], 0.0f, 0.0f, 0.0f, 0.0f);
-          else mma_bf16(c[nb], av, wb[ks][nb], c[nb][0], c[nb][1], c[nb][2], c[nb][3]);
-        }
-      } else {
-        // left pixels' columns without slot KS, right pixels' without slot
-        // 0: two products, each kept by the threads of its pixel
-        uint32_t al[4], ar[4];
+      for (int k = 0; k < KS * KS; ++k) {
+        float2 w[4];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int pi = ks * 8 + q + 4 * h, wi = pi % PR;
-          const uint32_t ml = pi >= PAIRS ? 0u : wi == PR - 1 ? 0x0000ffffu : 0xffffffffu;
-          const uint32_t mr = pi >= PAIRS ? 0u : wi == 0 ? 0xffff0000u : 0xffffffffu;
+        for (int j = 0; j < 4; j += 2)
+          asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                       : "=f"(w[j].x), "=f"(w[j].y), "=f"(w[j + 1].x), "=f"(w[j + 1].y)
+                       : "r"(w_addr + 4u * (uint32_t)(k * kClCout + ch0 + 2 * j)));
 #pragma unroll
-          for (int r = 0; r < 2; ++r) {
-            al[2 * h + r] = av[2 * h + r] & ml;
-            ar[2 * h + r] = av[2 * h + r] & mr;
+        for (int r = 0; r < 2; ++r)
+#pragma unroll
+          for (int j = 0; j < 4; ++j) cur[r][j] = fma2(f2(x[r + k / KS][k % KS]), w[j], cur[r][j]);
+      }
+    } else {
+      constexpr bool MASK = decltype(mask)::value;
+      uint32_t av[KSTEPS][4];
+#pragma unroll
+      for (int ks = 0; ks < KSTEPS; ++ks)
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int r = 0; r < 2; ++r)  // a0: (upper row, h 0), a1: (lower, 0), a2: (upper, 1), ...
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(av[ks][2 * h + r]) : "r"(p0 + aoff[ks][h] + r * row_b));
+#pragma unroll
+      for (int nb = 0; nb < 4; ++nb) {
+        float d[KSTEPS][4];
+#pragma unroll
+        for (int ks = 0; ks < KSTEPS; ++ks) {
+          if (!MASK) {
+            mma_bf16_zero(d[ks], av[ks], wb[ks][nb]);
+          } else {
+            // left pixels' columns without slot KS, right pixels' without slot
+            // 0: two products, each kept by the threads of its pixel
+            uint32_t al[4], ar[4];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              const int pi = ks * 8 + q + 4 * h, wi = pi % PR;
+              const uint32_t ml = pi >= PAIRS ? 0u : wi == PR - 1 ? 0x0000ffffu : 0xffffffffu;
+              const uint32_t mr = pi >= PAIRS ? 0u : wi == 0 ? 0xffff0000u : 0xffffffffu;
+#pragma unroll
+              for (int r = 0; r < 2; ++r) {
+                al[2 * h + r] = av[ks][2 * h + r] & ml;
+                ar[2 * h + r] = av[ks][2 * h + r] & mr;
+              }
+            }
+            float r[4];
+            mma_bf16_zero(d[ks], al, wb[ks][nb]);
+            mma_bf16_zero(r, ar, wb[ks][nb]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) d[ks][k] = right ? r[k] : d[ks][k];
           }
         }
 #pragma unroll
-        for (int nb = 0; nb < 4; ++nb) {
-          float l[4], r[4];
-          const bool z0 = ks == 0;
-          mma_bf16(l, al, wb[ks][nb], z0 ? 0.0f : c[nb][0], z0 ? 0.0f : c[nb][1], z0 ? 0.0f : c[nb][2],
-                   z0 ? 0.0f : c[nb][3]);
-          mma_bf16(r, ar, wb[ks][nb], z0 ? 0.0f : c[nb][0], z0 ? 0.0f : c[nb][1], z0 ? 0.0f : c[nb][2],
-                   z0 ? 0.0f : c[nb][3]);
-#pragma unroll
-          for (int k = 0; k < 4; ++k) c[nb][k] = right ? r[k] : l[k];
-        }
+        for (int r = 0; r < 2; ++r)
+          cur[r][nb] = add2(make_float2(d[0][2 * r], d[0][2 * r + 1]), make_float2(d[1][2 * r], d[1][2 * r + 1]));
       }
     }
     uint32_t zb[2];  // the 8 channels' spikes, upper and lower pixel
@@ -266,8 +314,7 @@ __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLea
       uint32_t zw[4], uw[4], acc = 0;
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const float2 un = leaky_pair<RESET>(beta[j], negthr[j], make_float2(c[j][2 * r], c[j][2 * r + 1]),
-                                            u[r][j], z[r][j]);
+        const float2 un = leaky_pair<RESET>(beta[j], negthr[j], cur[r][j], u[r][j], z[r][j]);
         uw[j] = Elem<__nv_bfloat16>::from2(un.x, un.y);
         zw[j] = Elem<__nv_bfloat16>::from2(z[r][j].x, z[r][j].y);
         acc |= (zw[j] & 0x00800080u) >> (7 - 2 * j);  // 1.0 is 0x3F80: bit 7 of each half
@@ -315,6 +362,11 @@ __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLea
     __syncthreads();  // these steps have landed; the other buffer is no longer read
     if (t0 + kClSteps < a.T) stage(t0 + kClSteps, buf ^ 1);
     const int n = min(kClSteps, a.T - t0);
+    const uint32_t p0 = sbase + (uint32_t)(buf * kClSteps * a.slice) + pix_addr;
+    if constexpr (!MMA) {  // a pixel's window alone: nothing to mask
+      for (int s = 0; s < n; ++s) step(p0 + (uint32_t)(s * a.slice), std::false_type());
+      continue;
+    }
     // an infinity or NaN among the staged pixels (elements of the slice past
     // the image were never written and are skipped): an exponent of all ones
     // plus one unit of it sets the half's top bit
@@ -327,7 +379,6 @@ __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLea
         odd |= ((x.x & e) + one) | ((x.y & e) + one) | ((x.z & e) + one) | ((x.w & e) + one);
       }
     }
-    const uint32_t p0 = sbase + (uint32_t)(buf * kClSteps * a.slice) + pix_addr;
     if (!__syncthreads_or(odd & 0x80008000u)) {
       for (int s = 0; s < n; ++s) step(p0 + (uint32_t)(s * a.slice), std::false_type());
     } else {
@@ -336,16 +387,23 @@ __global__ void __launch_bounds__(kClThreads, 8) conv_leaky_kernel(const ConvLea
   }
 }
 
+template <int KS, int RESET>
+cudaError_t launch_conv_leaky_reset(const ConvLeakyArgs& a, unsigned grid, size_t smem, cudaStream_t st) {
+  const auto kernel = conv_leaky_kernel<KS, RESET>;
+  if (smem > 48 * 1024) {
+    const cudaError_t e = ensure_smem((const void*)kernel, smem);
+    if (e != cudaSuccess) return e;
+  }
+  return launch_pdl(kernel, dim3(grid), dim3(kClThreads), smem, st, a);
+}
+
 template <int KS>
 cudaError_t launch_conv_leaky(const ConvLeakyArgs& a, int reset, unsigned grid, size_t smem,
                               cudaStream_t st) {
   switch (reset) {
-    case RESET_SUBTRACT:
-      return launch_pdl(conv_leaky_kernel<KS, RESET_SUBTRACT>, dim3(grid), dim3(kClThreads), smem, st, a);
-    case RESET_ZERO:
-      return launch_pdl(conv_leaky_kernel<KS, RESET_ZERO>, dim3(grid), dim3(kClThreads), smem, st, a);
-    default:
-      return launch_pdl(conv_leaky_kernel<KS, RESET_NONE>, dim3(grid), dim3(kClThreads), smem, st, a);
+    case RESET_SUBTRACT: return launch_conv_leaky_reset<KS, RESET_SUBTRACT>(a, grid, smem, st);
+    case RESET_ZERO: return launch_conv_leaky_reset<KS, RESET_ZERO>(a, grid, smem, st);
+    default: return launch_conv_leaky_reset<KS, RESET_NONE>(a, grid, smem, st);
   }
 }
 
@@ -411,8 +469,9 @@ extern "C" snn_status_t snn_conv2d_small_leaky_fwd_nhwc(
   int64_t rows = 2 * ((8 * kClWarps + Wp - 2) / Wp + 1) + KH - 1;
   if (rows > H) rows = H;
   a.slice = (int)(((rows * W + 8) * 2 + 15) / 16 * 16);  // + 8 elements for the start's round-down
-  const size_t smem = (size_t)2 * kClSteps * a.slice;
+  size_t smem = (size_t)2 * kClSteps * a.slice;
   if (smem > 48 * 1024 || d->B * parts > INT_MAX) return SNN_ERR_UNSUPPORTED;
+  if (KH == 3) smem += (size_t)(KH * KW * Cout) * sizeof(float);  // and the filters
   cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
   const unsigned grid = (unsigned)(d->B * parts);
   cudaError_t e;
