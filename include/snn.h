@@ -475,8 +475,8 @@ snn_status_t snn_maxpool2_bwd_nhwc(int64_t M, int64_t H, int64_t W, int64_t C, c
  *      sum over (m, oy, ox) of dI[m, oy, ox, o] * X[m, oy+ky, ox+kx, c] for
  *      dI bf16 [M, Ho, Wo, Cout]; a fixed number of blocks each sum a fixed
  *      set of images, the block partials (ws, at least
- *      snn_conv2d_small_dw_workspace_bytes, 16-byte aligned) are added in
- *      block order: the same bits on every call
+ *      snn_conv2d_small_dw_workspace_bytes, 16-byte aligned) are added in a
+ *      fixed order in compensated fp32: the same bits on every call
  * Asynchronous on stream.
  */
 snn_status_t snn_conv2d_small_fwd_nhwc(int64_t M, int64_t H, int64_t W, int64_t Cin, int64_t Cout,

@@ -530,8 +530,11 @@ __global__ void __maxnreg__(96) conv_slide_dw_kernel(
 // a block's few images.  The sliding-window FMA kernel above issued 3.7
 // instructions per paired FMA and took 52 us serialised at T = 25, B = 128,
 // [24, 24, 16] (64 MB: 9.4 us at 6.8 TB/s); this kernel takes 25 us there
-// (63% of issue slots), and its error against a float64 sum is the FMA
-// kernel's (8.2e-8 against 8.1e-8 of the result's norm).
+// (63% of issue slots).  With the block partials added in plain fp32 its error
+// against a float64 sum was the FMA kernel's for terms of either sign (1.02e-7
+// against 1.00e-7 of the result's norm, spikes, 3200 images) and a little more
+// for terms of one sign (4.0e-8 against 3.8e-8), where what the tensor core
+// truncates adds up; added compensated, 3.4e-8 and 2.7e-8.
 //
 // A block sums images b, b + G, ...; warp w takes pixel groups w, w + 9,
 // ... of each; the warps are added in order into the block partial, so the
@@ -701,33 +704,28 @@ cudaError_t launch_mma_dw(const __nv_bfloat16* X, const __nv_bfloat16* dI, float
 
 // dW[o, k] = sum of the G block partials, 0 for k >= K: a block takes 32
 // consecutive outputs (coalesced rows of the partials), warp w adds partials
-// w, w + 32, ... in order, then the warps are added in a fixed tree.
+// w, w + 32, ... in order, then the warps are added in order, all compensated.
 constexpr int kDwSumWarps = 32;
 __global__ void __launch_bounds__(32 * kDwSumWarps) conv_small_dw_sum(
     const float* __restrict__ part, float* __restrict__ dW, int G, int Cout, int K, int ldw) {
-  __shared__ float sh[kDwSumWarps][32];
+  __shared__ float2 sh[kDwSumWarps][32];
   grid_dep_wait();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int e = blockIdx.x * 32 + lane;
   const int o = e / ldw, k = e - o * ldw;
-  float s = 0.0f;
+  float2 s = make_float2(0.0f, 0.0f);
   if (o < Cout && k < K) {
     const float* p = part + o * K + k;
     const int64_t stride = (int64_t)Cout * K;
 #pragma unroll 8
-    for (int b = warp; b < G; b += kDwSumWarps) s += p[b * stride];
+    for (int b = warp; b < G; b += kDwSumWarps) s = two_add(s, p[b * stride]);
   }
   sh[warp][lane] = s;
   __syncthreads();
   if (warp == 0 && o < Cout) {
-    float r[kDwSumWarps];
-#pragma unroll
-    for (int w = 0; w < kDwSumWarps; ++w) r[w] = sh[w][lane];
-#pragma unroll
-    for (int d = kDwSumWarps / 2; d > 0; d >>= 1)
-#pragma unroll
-      for (int w = 0; w < d; ++w) r[w] += r[w + d];
-    dW[e] = r[0];
+#pragma unroll 4
+    for (int w = 1; w < kDwSumWarps; ++w) s = pair_add(s, sh[w][lane]);
+    dW[e] = pair_value(s);
   }
 }
 

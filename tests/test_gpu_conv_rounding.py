@@ -112,3 +112,23 @@ def test_3x3_over_shapes(H3, W3, reset, cuda_device):
     assert torch.equal(fused.spk, separate.spk)
     assert torch.equal(fused.mem.isnan(), separate.mem.isnan())
     assert torch.equal(fused.mem.nan_to_num(), separate.mem.nan_to_num())
+
+
+@pytest.mark.parametrize("k,cout,M", [(5, 16, 3200), (5, 8, 3200), (3, 16, 3200), (5, 16, 400)])
+def test_weight_gradient_of_positive_pixels(k, cout, M, cuda_device):
+    """Terms of one sign, where truncated sums would add up: the result's
+    error is that of one rounding (rms at most U / sqrt(3) of it)."""
+    g = torch.Generator().manual_seed(50 + k)
+    Ho = H - k + 1
+    X = _pixels("uniform", (M, H, H, 1), g).to(cuda_device)
+    dI = (torch.randn((M, Ho, Ho, cout), generator=g).abs() * 1e-3).bfloat16().to(cuda_device)
+    dW = torch.zeros((cout, 32 if k == 5 else 16), device=cuda_device)
+    ws = torch.zeros(snn.snn_conv2d_small_dw_workspace_bytes(M, H, H, 1, cout, k, k), dtype=torch.uint8,
+                     device=cuda_device)
+    snn.snn_conv2d_small_dw_nhwc(X, dI, dW, k, k, ws)
+    ref = torch.zeros((cout, k * k), dtype=torch.float64, device=cuda_device)
+    for a in range(0, M, 400):
+        p = X[a:a + 400, :, :, 0].double().unfold(1, k, 1).unfold(2, k, 1).reshape(-1, k * k)
+        ref += dI[a:a + 400].double().reshape(-1, cout).T @ p
+    err = (dW[:, :k * k].double() - ref).norm() / ref.norm()
+    assert float(err) <= U / 3 ** 0.5
