@@ -29,9 +29,9 @@ inline bool many_lanes(int64_t L) {
   return device_info(&d) == cudaSuccess && L >= kPlainManyLanes * (int64_t)d.sms;
 }
 
-template <bool SYN, typename TI, typename TO, int RESET, bool REC, int VL, bool STRIPS, bool CK>
+template <bool SYN, typename TI, typename TO, int RESET, bool REC, int VL, bool CK>
 cudaError_t fwd_staged_ck(ScanArgs a, cudaStream_t st, bool* launched) {
-  const void* k = (const void*)scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, STRIPS, CK>;
+  const void* k = (const void*)scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, CK>;
   StagedPlan p;
   // a stage holds kFwdRows steps of the strip's input row; one CTA per SM
   // where it fits (the longer rows stream faster), two for short sequences
@@ -44,28 +44,32 @@ cudaError_t fwd_staged_ck(ScanArgs a, cudaStream_t st, bool* launched) {
   a.stages = p.stages;
   a.stage_bytes = p.stage_bytes;
   *launched = true;
-  const int64_t grid = STRIPS && p.resident < p.grid ? p.resident : p.grid;
-  return launch_pdl(scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, STRIPS, CK>, dim3((unsigned)grid),
+  return launch_pdl(scan_fwd_staged<SYN, TI, TO, RESET, REC, VL, CK>, dim3((unsigned)p.grid),
                     dim3(p.threads), p.smem, st, a);
 }
 
-template <bool SYN, typename TI, typename TO, int RESET, bool REC, int VL, bool STRIPS>
+template <bool SYN, typename TI, typename TO, int RESET, bool REC, int VL>
 cudaError_t fwd_staged_vl(ScanArgs a, cudaStream_t st, bool* launched) {
-  return a.ckpt ? fwd_staged_ck<SYN, TI, TO, RESET, REC, VL, STRIPS, true>(a, st, launched)
-                : fwd_staged_ck<SYN, TI, TO, RESET, REC, VL, STRIPS, false>(a, st, launched);
+  return a.ckpt ? fwd_staged_ck<SYN, TI, TO, RESET, REC, VL, true>(a, st, launched)
+                : fwd_staged_ck<SYN, TI, TO, RESET, REC, VL, false>(a, st, launched);
 }
 
-// Short sequences (T <= 64) take 4 lanes a thread and CTAs that walk their
-// strips: with one CTA per strip each wave paid the ring's fill and drain
-// (T = 25, 128 x 6912 lanes in fp32, both passes: 127 us with 8 lanes and
-// three waves, 98 us so; 78 us at 6.8 TB/s).  Longer ones take 8 lanes
-// (Leaky; T = 500, 64 x 8192 lanes: 9% faster than 4 in store mode) unless
-// the lanes are few (T = 100, 64 x 4096: 20% slower than 4).
+// 4 lanes a thread instead of 8 (Leaky) with few lanes, which then make more
+// warps (T = 64, 128 x 1000 lanes in bf16: 9.4 us against 12.9; T = 100, 64 x
+// 4096: 20% faster), and for short sequences of fp32 currents (T = 25, 128 x
+// 6912 lanes: 43.9 us against 55.2).  Longer ones are better with 8 (T = 500,
+// 64 x 8192 lanes, store mode: 9% faster), and so are many lanes of short half
+// sequences (T = 10, 6.7 M lanes, recompute: 60.8 us against 68.8).  CTAs that
+// walk several strips with one ring were up to a fifth faster around 0.5 M
+// lanes (T = 25, fp32 recompute: 16.5 us against 20.1) but slower for many
+// (T = 1, 67 M lanes in bf16: 636 us against 291; T = 25, 128 x 6912 Synaptic
+// lanes: 64.5 against 58.8), so a CTA takes one.
 template <bool SYN, typename TI, typename TO, int RESET, bool REC = false>
 cudaError_t fwd_staged(ScanArgs a, cudaStream_t st, bool* launched) {
-  if (a.T <= 64) return fwd_staged_vl<SYN, TI, TO, RESET, REC, 4, true>(a, st, launched);
-  if (!SYN && few_lanes(a.L)) return fwd_staged_vl<SYN, TI, TO, RESET, REC, 4, false>(a, st, launched);
-  return fwd_staged_vl<SYN, TI, TO, RESET, REC, kLanes<SYN>, false>(a, st, launched);
+  if constexpr (!SYN)
+    if (few_lanes(a.L) || (a.T <= 64 && sizeof(TI) == 4))
+      return fwd_staged_vl<SYN, TI, TO, RESET, REC, 4>(a, st, launched);
+  return fwd_staged_vl<SYN, TI, TO, RESET, REC, kLanes<SYN>>(a, st, launched);
 }
 
 template <bool SYN, typename TI, typename TO, int RESET, int REC>

@@ -64,8 +64,7 @@ struct StagedPlan {
   int stages = 0;
   int stage_bytes = 0;
   size_t smem = 0;
-  int64_t grid = 0;      // strips
-  int64_t resident = 0;  // CTAs that run at once
+  int64_t grid = 0;
 };
 
 // Choose a staged launch for L lanes: all CTAs of a wave resident at once
@@ -128,7 +127,6 @@ inline bool plan_staged(const void* kernel, int64_t L, int64_t items, int stage_
       p.stage_bytes = (int)stage_bytes;
       p.smem = (size_t)(kBarrierBytes + stages * stage_bytes + seg_bytes);
       p.grid = ceil_div(L, lpc);
-      p.resident = (int64_t)d.sms * cps;
       if (ensure_smem(kernel, p.smem) != cudaSuccess) continue;
       int nb = 0;
       if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, p.smem) != cudaSuccess)

@@ -6,8 +6,7 @@
 // in t: each thread owns 8 or 4 consecutive lanes and keeps their state (u, i,
 // z and, backward, the adjoints) in registers for the whole scan.
 //
-// Staged kernels (the fast path): a CTA owns a contiguous strip of lanes, or
-// walks several (short sequences).
+// Staged kernels (the fast path): a CTA owns a contiguous strip of lanes.
 // One producer thread streams the strip's row of every input tensor, a few
 // steps at a time, into a ring of shared-memory stages with 1-D bulk copies (TMA,
 // cp.async.bulk) completing on a "full" mbarrier per stage; the consumer
@@ -618,17 +617,14 @@ __device__ __forceinline__ void store_partials(const ScanArgs& a, float* part, i
 // release per kFwdRows steps instead of per step.
 constexpr int kFwdRows = 8;
 
-// VL: lanes per thread.  STRIPS: a CTA walks the strips blockIdx.x, blockIdx.x
-// + gridDim.x, ... (else the grid has one CTA per strip): the ring runs on
-// across strips, so the next strip's rows arrive while the last steps of the
-// current one are computed.
+// VL: lanes per thread.
 // CK: checkpoints may be due (the recompute mode).  Without them a whole
 // stage is kFwdRows steps with no test in them, and the spike bits are taken
 // from the packed spikes (with the tests, 28 instructions a neuron-step: the
 // recurrent neuron's forward at T = 100 over 64 x 4096 lanes in bf16 took 38
 // us, so 31; 23 us at 6.8 TB/s).
 template <bool SYN, typename TI, typename TO, int RESET, bool REC = false, int VL = kLanes<SYN>,
-          bool STRIPS = false, bool CK = true>
+          bool CK = true>
 __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanArgs a) {
   constexpr int V = VL, NP = V / 2, R = kFwdRows;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -638,6 +634,8 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanA
   const int S = a.stages;
   const int cwarps = (int)(blockDim.x >> 5) - 1;
   const int warp = threadIdx.x >> 5, lid = threadIdx.x & 31;
+  const int64_t lane0 = (int64_t)blockIdx.x * a.lanes_per_cta;
+  const int cta_lanes = (int)min((int64_t)a.lanes_per_cta, a.L - lane0);
   const int row_elems = a.lanes_per_cta;  // a stage holds R rows of the strip
   init_ring_barriers(full, empty, S, cwarps);
   grid_dep_wait();  // the previous kernel on the stream is complete
@@ -646,18 +644,13 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanA
     if (lid == 0 && !(a.debug & DEBUG_PRODUCER_IDLE)) {
       Producer p{ring, full, empty, S, a.stage_bytes};
       const uint32_t row_bytes = (uint32_t)row_elems * (uint32_t)sizeof(TI);
-      for (int64_t lane0 = (int64_t)blockIdx.x * a.lanes_per_cta; lane0 < a.L && p.ok;
-           lane0 += (int64_t)gridDim.x * a.lanes_per_cta) {
-        const int cta_lanes = (int)min((int64_t)a.lanes_per_cta, a.L - lane0);
-        const uint32_t bytes = (uint32_t)cta_lanes * (uint32_t)sizeof(TI);
-        const TI* src = static_cast<const TI*>(a.I) + lane0;
-        for (int64_t t0 = 0; t0 < a.T; t0 += R) {
-          const int nr = (int)min((int64_t)R, a.T - t0);
-          if (!p.begin((uint32_t)nr * bytes, a)) break;
-          for (int r = 0; r < nr; ++r) p.copy((uint32_t)r * row_bytes, src + (t0 + r) * a.L, bytes);
-          p.end();
-        }
-        if (!STRIPS) break;
+      const uint32_t bytes = (uint32_t)cta_lanes * (uint32_t)sizeof(TI);
+      const TI* src = static_cast<const TI*>(a.I) + lane0;
+      for (int64_t t0 = 0; t0 < a.T; t0 += R) {
+        const int nr = (int)min((int64_t)R, a.T - t0);
+        if (!p.begin((uint32_t)nr * bytes, a)) break;
+        for (int r = 0; r < nr; ++r) p.copy((uint32_t)r * row_bytes, src + (t0 + r) * a.L, bytes);
+        p.end();
       }
       p.drain();
     }
@@ -668,158 +661,153 @@ __global__ void __launch_bounds__(kMaxStagedThreads) scan_fwd_staged(const ScanA
   const TI* my = reinterpret_cast<const TI*>(ring) + c * V;
   const int stage_elems = a.stage_bytes / (int)sizeof(TI);
   RingPos pos;
-  for (int64_t lane0 = (int64_t)blockIdx.x * a.lanes_per_cta; lane0 < a.L;
-       lane0 += (int64_t)gridDim.x * a.lanes_per_cta) {
-    const int cta_lanes = (int)min((int64_t)a.lanes_per_cta, a.L - lane0);
-    const int64_t l = lane0 + (int64_t)c * V;
-    const bool active = c * V < cta_lanes;
-    float2 beta[NP], negthr[NP], third[NP], u[NP], z[NP], in[NP];
-    if (active) {
-      load_params<SYN || REC, NP>(a, l, beta, negthr, third);
-      bool zb[V];
-      initial_state<SYN, NP>(a, l, negthr, u, zb, in);
+  const int64_t l = lane0 + (int64_t)c * V;
+  const bool active = c * V < cta_lanes;
+  float2 beta[NP], negthr[NP], third[NP], u[NP], z[NP], in[NP];
+  if (active) {
+    load_params<SYN || REC, NP>(a, l, beta, negthr, third);
+    bool zb[V];
+    initial_state<SYN, NP>(a, l, negthr, u, zb, in);
 #pragma unroll
-      for (int k = 0; k < NP; ++k) {
-        z[k] = make_float2(zb[2 * k] ? 1.0f : 0.0f, zb[2 * k + 1] ? 1.0f : 0.0f);
-        if (REC) third[k] = add2_rn(third[k], negthr[k]);  // v - thr, rounded once
-      }
+    for (int k = 0; k < NP; ++k) {
+      z[k] = make_float2(zb[2 * k] ? 1.0f : 0.0f, zb[2 * k + 1] ? 1.0f : 0.0f);
+      if (REC) third[k] = add2_rn(third[k], negthr[k]);  // v - thr, rounded once
     }
-    TO* spk = static_cast<TO*>(a.spk) + l;
-    TO* mem = a.mem ? static_cast<TO*>(a.mem) + l : nullptr;
-    TO* syn = (SYN && a.syn) ? static_cast<TO*>(a.syn) + l : nullptr;
-    float* ck = a.ckpt ? a.ckpt + l : nullptr;
-    const int64_t ck_stride = SYN ? 2 * a.L : a.L;
-    // spike bits: one byte per thread and step (8 lanes), or one per pair of
-    // threads (4 lanes each: the even thread stores)
-    unsigned char* bits = a.bits ? a.bits + lane0 / 8 + (V == 4 ? c / 2 : c) : nullptr;
-    int kk = a.nseg > 0 ? seg_phase0(a) : 0;  // position inside the current checkpoint segment
-    for (int64_t t0 = 0; t0 < a.T; t0 += R) {
-      if (!warp_wait(&full[pos.s], pos.ph, a.wait_ns)) {
-        if (lid == 0) record_status(a.status, kStatusTimeout);
-        return;
-      }
-      const int nr = (int)min((int64_t)R, a.T - t0);
-      if constexpr (!CK) {
-        uint32_t nibs = 0;  // V == 4: the thread's four spikes of step r at bit 4*r
-        auto step = [&](const TI* x_row, TO* spk_row, TO* mem_row, TO* syn_row, unsigned char* bit_byte,
-                        int r) {
-          float2 x[NP];
-          load_pairs<TI, NP>(x_row, x);
+  }
+  TO* spk = static_cast<TO*>(a.spk) + l;
+  TO* mem = a.mem ? static_cast<TO*>(a.mem) + l : nullptr;
+  TO* syn = (SYN && a.syn) ? static_cast<TO*>(a.syn) + l : nullptr;
+  float* ck = a.ckpt ? a.ckpt + l : nullptr;
+  const int64_t ck_stride = SYN ? 2 * a.L : a.L;
+  // spike bits: one byte per thread and step (8 lanes), or one per pair of
+  // threads (4 lanes each: the even thread stores)
+  unsigned char* bits = a.bits ? a.bits + lane0 / 8 + (V == 4 ? c / 2 : c) : nullptr;
+  int kk = a.nseg > 0 ? seg_phase0(a) : 0;  // position inside the current checkpoint segment
+  for (int64_t t0 = 0; t0 < a.T; t0 += R) {
+    if (!warp_wait(&full[pos.s], pos.ph, a.wait_ns)) {
+      if (lid == 0) record_status(a.status, kStatusTimeout);
+      return;
+    }
+    const int nr = (int)min((int64_t)R, a.T - t0);
+    if constexpr (!CK) {
+      uint32_t nibs = 0;  // V == 4: the thread's four spikes of step r at bit 4*r
+      auto step = [&](const TI* x_row, TO* spk_row, TO* mem_row, TO* syn_row, unsigned char* bit_byte,
+                      int r) {
+        float2 x[NP];
+        load_pairs<TI, NP>(x_row, x);
 #pragma unroll
-          for (int k = 0; k < NP; ++k)
-            fwd_pair<SYN, RESET, REC ? 1 : 0>(a.reset, beta[k], negthr[k], third[k], x[k], u[k], z[k], in[k]);
-          if constexpr (sizeof(TO) == 2) {
-            uint32_t w[NP];
+        for (int k = 0; k < NP; ++k)
+          fwd_pair<SYN, RESET, REC ? 1 : 0>(a.reset, beta[k], negthr[k], third[k], x[k], u[k], z[k], in[k]);
+        if constexpr (sizeof(TO) == 2) {
+          uint32_t w[NP];
 #pragma unroll
-            for (int k = 0; k < NP; ++k) w[k] = Elem<TO>::from2(z[k].x, z[k].y);
-            if constexpr (V == 8) *reinterpret_cast<uint4*>(spk_row) = make_uint4(w[0], w[1], w[2], w[3]);
-            else *reinterpret_cast<uint2*>(spk_row) = make_uint2(w[0], w[1]);
-            if (bits) {
-              // one set bit of 1.0's exponent per half: bf16 0x3F80, fp16 0x3C00
-              constexpr uint32_t one = std::is_same<TO, __half>::value ? 0x04000400u : 0x00800080u;
-              constexpr int at = std::is_same<TO, __half>::value ? 10 : 7;
-              uint32_t t = 0;
+          for (int k = 0; k < NP; ++k) w[k] = Elem<TO>::from2(z[k].x, z[k].y);
+          if constexpr (V == 8) *reinterpret_cast<uint4*>(spk_row) = make_uint4(w[0], w[1], w[2], w[3]);
+          else *reinterpret_cast<uint2*>(spk_row) = make_uint2(w[0], w[1]);
+          if (bits) {
+            // one set bit of 1.0's exponent per half: bf16 0x3F80, fp16 0x3C00
+            constexpr uint32_t one = std::is_same<TO, __half>::value ? 0x04000400u : 0x00800080u;
+            constexpr int at = std::is_same<TO, __half>::value ? 10 : 7;
+            uint32_t t = 0;
 #pragma unroll
-              for (int k = 0; k < NP; ++k) t |= ((w[k] & one) >> at) << (2 * k);
-              t = (t | (t >> 15)) & ((1u << V) - 1u);
-              if constexpr (V == 8) *bit_byte = (unsigned char)t;
-              else nibs |= t << (4 * r);
-            }
-          } else {
-            store_pairs<TO, NP>(spk_row, z);
+            for (int k = 0; k < NP; ++k) t |= ((w[k] & one) >> at) << (2 * k);
+            t = (t | (t >> 15)) & ((1u << V) - 1u);
+            if constexpr (V == 8) *bit_byte = (unsigned char)t;
+            else nibs |= t << (4 * r);
           }
-          if (mem) store_pairs<TO, NP>(mem_row, u);
-          if (SYN && syn) store_pairs<TO, NP>(syn_row, in);
-        };
-        if (active) {
-          const TI* st = my + pos.s * stage_elems;
-          const int64_t L = a.L;
-          if (nr == R) {
+        } else {
+          store_pairs<TO, NP>(spk_row, z);
+        }
+        if (mem) store_pairs<TO, NP>(mem_row, u);
+        if (SYN && syn) store_pairs<TO, NP>(syn_row, in);
+      };
+      if (active) {
+        const TI* st = my + pos.s * stage_elems;
+        const int64_t L = a.L;
+        if (nr == R) {
 #pragma unroll
-            for (int r = 0; r < R; ++r)
-              step(st + r * row_elems, spk + r * L, mem + r * L, syn + r * L, bits + r * a.bits_row, r);
-          } else {
+          for (int r = 0; r < R; ++r)
+            step(st + r * row_elems, spk + r * L, mem + r * L, syn + r * L, bits + r * a.bits_row, r);
+        } else {
 #pragma unroll 1
-            for (int r = 0; r < nr; ++r)
-              step(st + r * row_elems, spk + r * L, mem + r * L, syn + r * L, bits + r * a.bits_row, r);
-          }
-        }
-        if (bits) {
-          if constexpr (V == 4) {
-            // a byte's halves sit in neighbouring threads: the even one stores
-            // the stage's first four steps, the odd one the others
-            const uint32_t other = __shfl_xor_sync(0xffffffffu, nibs, 1);
-            const int odd = c & 1;
-            const uint32_t lo = (odd ? other : nibs) >> (16 * odd), hi = (odd ? nibs : other) >> (16 * odd);
-#pragma unroll
-            for (int k = 0; k < R / 2; ++k)
-              if (active && k + odd * (R / 2) < nr)
-                bits[(k + odd * (R / 2)) * a.bits_row] =
-                    (unsigned char)(((lo >> (4 * k)) & 15u) | (((hi >> (4 * k)) & 15u) << 4));
-          }
-          bits += R * a.bits_row;
-        }
-      } else {
-        unsigned zbits[R];
-        if (active) {
-          const TI* st = my + pos.s * stage_elems;
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            zbits[r] = 0;
-            if (r < nr) {
-              float2 x[NP];
-              load_pairs<TI, NP>(st + r * row_elems, x);
-#pragma unroll
-              for (int k = 0; k < NP; ++k)
-                fwd_pair<SYN, RESET, REC ? 1 : 0>(a.reset, beta[k], negthr[k], third[k], x[k], u[k],
-                                                  z[k], in[k]);
-              if (bits) {
-#pragma unroll
-                for (int k = 0; k < NP; ++k) {
-                  zbits[r] |= ((z[k].x != 0.0f) ? 1u : 0u) << (2 * k);
-                  zbits[r] |= ((z[k].y != 0.0f) ? 1u : 0u) << (2 * k + 1);
-                }
-              }
-              store_pairs<TO, NP>(spk + r * a.L, z);
-              if (mem) store_pairs<TO, NP>(mem + r * a.L, u);
-              if (SYN && syn) store_pairs<TO, NP>(syn + r * a.L, in);
-              if (++kk == a.K) {
-                kk = 0;
-                if (ck && t0 + r + 1 < a.T) {
-                  store_pairs<float, NP>(ck, u);
-                  if (SYN) store_pairs<float, NP>(ck + a.L, in);
-                  ck += ck_stride;
-                }
-              }
-            }
-          }
-        }
-        if (bits) {
-#pragma unroll
-          for (int r = 0; r < R; ++r) {
-            if (r < nr) {
-              if (V == 4) {
-                const unsigned hi = __shfl_down_sync(0xffffffffu, zbits[r], 1);
-                if (active && !(c & 1)) bits[r * a.bits_row] = (unsigned char)(zbits[r] | (hi << 4));
-              } else if (active) {
-                bits[r * a.bits_row] = (unsigned char)zbits[r];
-              }
-            }
-          }
-          bits += R * a.bits_row;
+          for (int r = 0; r < nr; ++r)
+            step(st + r * row_elems, spk + r * L, mem + r * L, syn + r * L, bits + r * a.bits_row, r);
         }
       }
-      release_stage(empty, pos.s, lid);
-      pos.next(S);
-      spk += R * a.L;
-      if (mem) mem += R * a.L;
-      if (SYN && syn) syn += R * a.L;
+      if (bits) {
+        if constexpr (V == 4) {
+          // a byte's halves sit in neighbouring threads: the even one stores
+          // the stage's first four steps, the odd one the others
+          const uint32_t other = __shfl_xor_sync(0xffffffffu, nibs, 1);
+          const int odd = c & 1;
+          const uint32_t lo = (odd ? other : nibs) >> (16 * odd), hi = (odd ? nibs : other) >> (16 * odd);
+#pragma unroll
+          for (int k = 0; k < R / 2; ++k)
+            if (active && k + odd * (R / 2) < nr)
+              bits[(k + odd * (R / 2)) * a.bits_row] =
+                  (unsigned char)(((lo >> (4 * k)) & 15u) | (((hi >> (4 * k)) & 15u) << 4));
+        }
+        bits += R * a.bits_row;
+      }
+    } else {
+      unsigned zbits[R];
+      if (active) {
+        const TI* st = my + pos.s * stage_elems;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          zbits[r] = 0;
+          if (r < nr) {
+            float2 x[NP];
+            load_pairs<TI, NP>(st + r * row_elems, x);
+#pragma unroll
+            for (int k = 0; k < NP; ++k)
+              fwd_pair<SYN, RESET, REC ? 1 : 0>(a.reset, beta[k], negthr[k], third[k], x[k], u[k],
+                                                z[k], in[k]);
+            if (bits) {
+#pragma unroll
+              for (int k = 0; k < NP; ++k) {
+                zbits[r] |= ((z[k].x != 0.0f) ? 1u : 0u) << (2 * k);
+                zbits[r] |= ((z[k].y != 0.0f) ? 1u : 0u) << (2 * k + 1);
+              }
+            }
+            store_pairs<TO, NP>(spk + r * a.L, z);
+            if (mem) store_pairs<TO, NP>(mem + r * a.L, u);
+            if (SYN && syn) store_pairs<TO, NP>(syn + r * a.L, in);
+            if (++kk == a.K) {
+              kk = 0;
+              if (ck && t0 + r + 1 < a.T) {
+                store_pairs<float, NP>(ck, u);
+                if (SYN) store_pairs<float, NP>(ck + a.L, in);
+                ck += ck_stride;
+              }
+            }
+          }
+        }
+      }
+      if (bits) {
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (r < nr) {
+            if (V == 4) {
+              const unsigned hi = __shfl_down_sync(0xffffffffu, zbits[r], 1);
+              if (active && !(c & 1)) bits[r * a.bits_row] = (unsigned char)(zbits[r] | (hi << 4));
+            } else if (active) {
+              bits[r * a.bits_row] = (unsigned char)zbits[r];
+            }
+          }
+        }
+        bits += R * a.bits_row;
+      }
     }
-    if (active) {
-      if (a.mem_final) store_pairs<float, NP>(a.mem_final + l, u);
-      if (SYN && a.syn_final) store_pairs<float, NP>(a.syn_final + l, in);
-    }
-    if (!STRIPS) break;
+    release_stage(empty, pos.s, lid);
+    pos.next(S);
+    spk += R * a.L;
+    if (mem) mem += R * a.L;
+    if (SYN && syn) syn += R * a.L;
+  }
+  if (active) {
+    if (a.mem_final) store_pairs<float, NP>(a.mem_final + l, u);
+    if (SYN && a.syn_final) store_pairs<float, NP>(a.syn_final + l, in);
   }
 }
 
