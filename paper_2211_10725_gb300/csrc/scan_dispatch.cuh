@@ -118,7 +118,13 @@ cudaError_t bwd_staged_vl(ScanArgs a, cudaStream_t st, bool* launched) {
     items = ceil_div(a.T, kBwdRows);
   }
   StagedPlan p;
-  if (!plan_staged(k, a.L, items, per_lane, seg, VL, &p, fixed, KC, 2, part_align(a))) return cudaSuccess;
+  // Short store-mode sequences may have a ring of two items (8 steps): asking
+  // for three made their strips narrower than the lanes of one wave, and the
+  // second wave cost more than the third item gives (us, T = 13, per-neuron
+  // parameters: 262,144 fp32 Synaptic lanes 18.8 -> 15.0, 524,288 fp32 Leaky
+  // lanes 22.7 -> 20.1; 4 M bf16 Leaky lanes 78 -> 82)
+  const int ring = !RECOMP && a.T <= 64 ? 2 : 3;
+  if (!plan_staged(k, a.L, items, per_lane, seg, VL, &p, fixed, KC, 2, part_align(a), ring)) return cudaSuccess;
   choose_parts(a, p, VL);
   a.lanes_per_cta = p.lanes_per_cta;
   a.stages = p.stages;

@@ -78,10 +78,11 @@ struct StagedPlan {
 //   force_stages: exact ring depth the kernel was compiled for (0 = any)
 //   max_cps: most CTAs per SM to try (larger strips first when 1)
 //   lane_align: the strips' lanes are a multiple of it (8, 16 or 32)
+//   ring: fewest stages (the caller passes the same for a kernel and item count)
 inline bool plan_staged(const void* kernel, int64_t L, int64_t items, int stage_bytes_per_lane,
                         int seg_bytes_per_thread, int lanes_per_thread, StagedPlan* plan,
                         int fixed_bytes_per_lane = 0, int force_stages = 0, int max_cps = 2,
-                        int lane_align = 8) {
+                        int lane_align = 8, int ring = 3) {
   static std::mutex mu;
   static std::map<std::tuple<int, const void*, int64_t, int64_t, int, int, int>, StagedPlan> cache;
   int dev = 0;
@@ -101,7 +102,7 @@ inline bool plan_staged(const void* kernel, int64_t L, int64_t items, int stage_
   if (device_info(&d) != cudaSuccess) return false;
   cudaFuncAttributes fa;
   if (cudaFuncGetAttributes(&fa, kernel) != cudaSuccess) return false;
-  const int min_stages = (int)(items < 3 ? (items < 1 ? 1 : items) : 3);
+  const int min_stages = (int)(items < ring ? (items < 1 ? 1 : items) : ring);
   for (int waves = 1; waves <= 64; ++waves) {
     for (int cps = max_cps; cps >= 1; --cps) {
       const int64_t ctas = (int64_t)d.sms * cps * waves;
