@@ -8,7 +8,7 @@
 // byte round trip and the spikes were read back for pooling.  At T = 25,
 // B = 128, 28x28 -> [24, 24, 16] (146 MB written: 21 us at 6.8 TB/s) the
 // three kernels took 48 + 45 + 12 us one at a time from a cold cache, this
-// one 30 us (61% of issue slots); with the weight gradient's product (see
+// one 30 us (58% of issue slots); with the weight gradient's product (see
 // conv_small.cu) the CSNN's training step went from 510 to 406 us.
 //
 // Mapping: a warp owns 8 pooled pixels (2x2 windows) for all T steps.  Per
